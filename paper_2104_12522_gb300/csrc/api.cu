@@ -69,6 +69,26 @@ bart_status bart_scratch(bart_ctx* ctx, const char* name, size_t bytes, void** o
   return BART_OK;
 }
 
+bart_status bart_scratch_any(bart_ctx* ctx, const char* name, size_t bytes, void** out, std::vector<void*>* held) {
+  auto it = ctx->scratch.find(name);
+  const bool fits = it != ctx->scratch.end() && it->second.second >= bytes;
+  if (fits || !stream_capturing(ctx)) return bart_scratch(ctx, name, bytes, out);
+  void* p = nullptr;
+  if (cudaMallocAsync(&p, bytes < 256 ? 256 : bytes, ctx->stream) != cudaSuccess) {
+    cudaGetLastError();
+    return bart_fail(ctx, BART_ENOMEM, "scratch '%s': %zu bytes could not be taken inside the capture", name, bytes);
+  }
+  held->push_back(p);
+  *out = p;
+  return BART_OK;
+}
+
+void bart_scratch_give_back(bart_ctx* ctx, std::vector<void*>* held) {
+  for (void* p : *held)
+    if (cudaFreeAsync(p, ctx->stream) != cudaSuccess) cudaGetLastError();
+  held->clear();
+}
+
 bart_status bart_upload_const(bart_ctx* ctx, const char* name, const void* data, size_t bytes, void** dev) {
   void* before = nullptr;
   auto it0 = ctx->scratch.find(name);

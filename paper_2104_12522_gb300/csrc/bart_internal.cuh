@@ -56,6 +56,14 @@ bart_status bart_fail(bart_ctx* ctx, bart_status st, const char* fmt, ...);
 // Scratch buffer of at least `bytes` bytes named `name`, kept for later calls.
 bart_status bart_scratch(bart_ctx* ctx, const char* name, size_t bytes, void** out);
 
+// Scratch for an entry point that may be called inside a stream capture without
+// an eager call before it: the kept buffer where it is large enough (or can
+// grow), else, while the stream is being captured, memory that the graph itself
+// allocates and frees.  Buffers of the second kind are listed in `held`;
+// bart_scratch_give_back frees them after the last launch that uses them.
+bart_status bart_scratch_any(bart_ctx* ctx, const char* name, size_t bytes, void** out, std::vector<void*>* held);
+void bart_scratch_give_back(bart_ctx* ctx, std::vector<void*>* held);
+
 // Device copy of a small host constant buffer, kept in scratch `name`.  The
 // copy is issued only when the bytes differ from the last upload, so a call
 // repeated with the same arguments launches kernels only (and can be captured
