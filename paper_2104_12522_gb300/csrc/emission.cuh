@@ -98,6 +98,20 @@ inline bool fused_offsets_fit(const bart_grid_desc* g) {
   return (int64_t)g->n_species * g->n_layers * g->n_temps * g->nu.n_nu + g->nu.n_nu <= (int64_t)UINT32_MAX;
 }
 
+// Checks shared by the batched forward model and the contribution functions.
+bart_status check_forward_request(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b);
+
+// Constants, layer brackets and abundance coefficients of an emission batch:
+// uploads the constant table and launches tp_kernel on the context's stream.
+struct EmPrep {
+  const float* dc;      // [p_cgs L][t_axis M][dpg L-1][ang 2NA][x0 S]
+  size_t off_dpg, off_ang;
+  LayerTW* tw;
+  float* coef;
+};
+bart_status emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
+                              EmPrep* out);
+
 // The persistent fused launch of an emission batch (forward_fused.cu).
 bart_status fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
                            float* spectra, const bart_filters* f, float* bands, int nb);

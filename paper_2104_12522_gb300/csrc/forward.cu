@@ -255,167 +255,6 @@ __global__ void band_integrate_kernel(const float* __restrict__ spectra, const i
   }
 }
 
-// Contribution functions of the emission spectrum (post-processing of
-// Sec. 3): the same layer loop as emission_kernel, one thread per (proposal,
-// wavenumber), but each layer's term of the intensity sum is stored instead
-// of accumulated: C_k = 2 pi sum_i w_i mu_i (B_k + B_{k+1})/2 (t_k - t_{k+1})
-// for the layer between levels k and k+1, then at the last level integrated
-// (kb: the deck, the optical-depth limit or L-1) its blackbody seen through
-// the column, and zeros below.  sum_k C_k is the flux of emission_kernel.
-// Species count and the Planck/limit options are runtime values here (a
-// post-processing pass over a few spectra), only the angle count is a
-// template parameter.
-constexpr int CF_THREADS = 128;
-
-template <int NA>
-__global__ void __launch_bounds__(CF_THREADS)
-contrib_kernel(const float* __restrict__ grid, int S, int L, int M, int64_t N, const LayerTW* __restrict__ tw,
-               const float* __restrict__ coef, const float* __restrict__ dpg, const float* __restrict__ ang,
-               double nu_start, double dnu, const int64_t* __restrict__ nu_lo, const int64_t* __restrict__ nu_hi,
-               float* __restrict__ contrib, const int32_t* __restrict__ act_mask, int* __restrict__ status,
-               EmExtra ex, int wide_x, int tau_lim) {
-  const int p = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (act_mask && !act_mask[p]) return;
-  const int64_t lo = nu_lo ? nu_lo[p] : 0;
-  const int64_t hi = nu_hi ? nu_hi[p] : N;
-  if (lo < 0 || hi > N || lo >= hi) {
-    if (tid == 0 && blockIdx.y == 0) atomicOr(status, BART_DEV_RANGE);
-    return;
-  }
-  const int64_t j = lo + (int64_t)blockIdx.y * CF_THREADS + tid;
-  if (j >= hi) return;                       // no block-level synchronisation below
-  float xs[4];
-  for (int s = 0; s < 4; ++s) xs[s] = s < S ? coef[(int64_t)p * S + s] : 0.0f;
-  const double nu = nu_start + (double)j * dnu;
-  const float nuf = (float)nu;
-  const float c1nu3 = (float)(2.0 * bartc::H * bartc::C * bartc::C * nu * nu * nu);
-  const float chi_r = (float)(ex.ray * (nu * nu) * (nu * nu));
-  float nl2mu[NA], wmu[NA], lt[NA], t[NA];
-#pragma unroll
-  for (int i = 0; i < NA; ++i) {
-    nl2mu[i] = ang[i];
-    wmu[i] = ang[NA + i];
-    lt[i] = 0.0f;
-    t[i] = 1.0f;
-  }
-  const LayerTW* twp = tw + (int64_t)p * L;
-  const int64_t sstride = (int64_t)L * M * N;
-  const int64_t dm = (M > 1) ? N : 0;
-  const float* gj = grid + j;
-  auto chi_at = [&](const LayerTW& r) {
-    float chi = chi_r;
-    for (int s = 0; s < S; ++s) {
-      const float a = __ldg(gj + r.row + s * sstride);
-      const float b = __ldg(gj + r.row + s * sstride + dm);
-      chi = fmaf(xs[s], fmaf(r.w, b - a, a), chi);
-    }
-    return chi;
-  };
-  auto planck_x = [&](float x) { return wide_x ? planck<true>(c1nu3, x) : planck<false>(c1nu3, x); };
-  float* out = contrib + (int64_t)p * L * N + j;
-  LayerTW r = twp[0];
-  float chi_prev = chi_at(r);
-  float B_prev = planck_x(nuf * r.c2_t);
-  float tau_v = 0.0f;
-  int k = 1;
-  for (; k < ex.L_run; ++k) {
-    r = twp[k];
-    const float chi = chi_at(r);
-    const float B = planck_x(nuf * r.c2_t);
-    const float dtau = (chi_prev + chi) * dpg[k - 1];
-    const float Bsum = B_prev + B;
-    float C = 0.0f;
-#pragma unroll
-    for (int i = 0; i < NA; ++i) {
-      lt[i] = fmaf(dtau, nl2mu[i], lt[i]);
-      const float te = bartf::ex2_approx(lt[i]);
-      C = fmaf(wmu[i], Bsum * (t[i] - te), C);
-      t[i] = te;
-    }
-    out[(int64_t)(k - 1) * N] = C;
-    chi_prev = chi;
-    B_prev = B;
-    if (tau_lim) {
-      tau_v += dtau;
-      if (tau_v > ex.tau_cut) {
-        ++k;
-        break;
-      }
-    }
-  }
-  // k - 1 is now the last level integrated: its blackbody through the column
-  float Cb = 0.0f;
-#pragma unroll
-  for (int i = 0; i < NA; ++i) Cb = fmaf(wmu[i], 2.0f * B_prev * t[i], Cb);
-  out[(int64_t)(k - 1) * N] = Cb;
-  for (int q = k; q < L; ++q) out[(int64_t)q * N] = 0.0f;
-}
-
-// Band means of contribution rows: one CTA per (row = proposal x level, band),
-// trapezoid weights over the proposal's span, FP64 sums (as
-// band_integrate_kernel).
-__global__ void contrib_band_kernel(const float* __restrict__ contrib, int L, int64_t N,
-                                    const int64_t* __restrict__ nu_lo, const int64_t* __restrict__ nu_hi,
-                                    const float* __restrict__ filt, int n_bands, const int32_t* __restrict__ act_mask,
-                                    float* __restrict__ out) {
-  const int row = blockIdx.x, b = blockIdx.y;
-  const int p = row / L;
-  if (act_mask && !act_mask[p]) return;
-  const int64_t lo = nu_lo ? nu_lo[p] : 0, hi = nu_hi ? nu_hi[p] : N;
-  if (lo < 0 || hi > N || lo >= hi) return;   // reported by contrib_kernel
-  const float* c = contrib + (int64_t)row * N;
-  double num = 0.0, den = 0.0;
-  for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-    const float dw = (hi - lo == 1) ? 1.0f : ((j == lo || j == hi - 1) ? 0.5f : 1.0f);
-    const float W = __ldg(filt + (int64_t)b * N + j) * dw;
-    num += (double)W * (double)c[j];
-    den += (double)W;
-  }
-  __shared__ double sn[32], sd[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    num += __shfl_xor_sync(0xffffffffu, num, o);
-    den += __shfl_xor_sync(0xffffffffu, den, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sn[threadIdx.x >> 5] = num;
-    sd[threadIdx.x >> 5] = den;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, d = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a += sn[w];
-      d += sd[w];
-    }
-    out[(int64_t)row * n_bands + b] = d > 0.0 ? (float)(a / d) : 0.0f;
-  }
-}
-
-using CfLauncher = void (*)(dim3, cudaStream_t, const float*, int, int, int, int64_t, const LayerTW*, const float*,
-                            const float*, const float*, double, double, const int64_t*, const int64_t*, float*,
-                            const int32_t*, int*, EmExtra, int, int);
-
-template <int NA>
-void launch_contrib(dim3 g, cudaStream_t st, const float* grid, int S, int L, int M, int64_t N, const LayerTW* tw,
-                    const float* coef, const float* dpg, const float* ang, double nu_start, double dnu,
-                    const int64_t* lo, const int64_t* hi, float* contrib, const int32_t* active, int* status,
-                    EmExtra ex, int wide_x, int tau_lim) {
-  contrib_kernel<NA><<<g, CF_THREADS, 0, st>>>(grid, S, L, M, N, tw, coef, dpg, ang, nu_start, dnu, lo, hi, contrib,
-                                               active, status, ex, wide_x, tau_lim);
-}
-
-CfLauncher pick_contrib(int na) {
-  switch (na) {
-    case 1: return launch_contrib<1>;
-    case 2: return launch_contrib<2>;
-    case 4: return launch_contrib<4>;
-    case 8: return launch_contrib<8>;
-    case 16: return launch_contrib<16>;
-    default: return nullptr;
-  }
-}
-
 template <int S, int NA, int TW, int MODE>
 void launch_emission(dim3 g, cudaStream_t st, const float* grid, int L, int M, int64_t N, const LayerTW* tw,
                      const float* coef, const float* dpg, const float* ang, double nu_start, double dnu,
@@ -550,10 +389,8 @@ int bartem::emission_mode(const bart_grid_desc* g, const bart_fwd_cfg* c) {
 bart_status bart_transmission_batch(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
                                     const bart_batch* b, float* spectra, const bart_filters* f, float* bands);
 
-namespace {
-
 // Checks shared by the batched forward model and the contribution functions.
-bart_status check_forward_request(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
+bart_status bartem::check_forward_request(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
                                   const bart_batch* b) {
   BART_REQUIRE(ctx, g && c && b, "NULL grid, cfg or batch");
   BART_REQUIRE(ctx, g->grid, "grid->grid is NULL");
@@ -577,16 +414,7 @@ bart_status check_forward_request(bart_ctx* ctx, const bart_grid_desc* g, const 
   return BART_OK;
 }
 
-// Constants, layer brackets and abundance coefficients of an emission batch:
-// uploads the constant table and launches tp_kernel on the context's stream.
-struct EmPrep {
-  const float* dc;      // [p_cgs L][t_axis M][dpg L-1][ang 2NA][x0 S]
-  size_t off_dpg, off_ang;
-  LayerTW* tw;
-  float* coef;
-};
-
-bart_status emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
+bart_status bartem::emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
                               EmPrep* out) {
   const int S = g->n_species, L = g->n_layers, M = g->n_temps, n = b->n;
   const int64_t N = g->nu.n_nu;
@@ -624,8 +452,6 @@ bart_status emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart
   out->coef = (float*)p_coef;
   return BART_OK;
 }
-
-}  // namespace
 
 extern "C" bart_status bart_forward_spectra_batch(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
                                                   const bart_batch* b, float* spectra, const bart_filters* f,
@@ -732,49 +558,6 @@ extern "C" bart_status bart_band_integrate(bart_ctx* ctx, const float* spectra, 
   band_integrate_kernel<<<grid_dim, 256, 0, ctx->stream>>>(spectra, spec_offsets, nu_lo, nu_hi, nu.n_nu,
                                                           f->weights, f->n_bands, out, ctx->d_status);
   return bart_check_launch(ctx, "band_integrate_kernel");
-}
-
-extern "C" bart_status bart_contribution_functions(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
-                                                   const bart_batch* b, float* contrib, const bart_filters* f,
-                                                   float* bands) {
-  if (!ctx) return BART_EINVAL;
-  bart_status st;
-  if ((st = check_forward_request(ctx, g, c, b)) != BART_OK) return st;
-  BART_REQUIRE(ctx, c->geometry == BART_EMISSION, "contribution functions are defined for emission only");
-  BART_REQUIRE(ctx, contrib || bands, "nothing requested: contrib and bands are both NULL");
-  int nb = 0;
-  if (bands) {
-    BART_REQUIRE(ctx, f && f->weights, "bands requested without filters");
-    nb = f->n_bands;
-    BART_REQUIRE(ctx, nb >= 1 && nb <= 65535, "n_bands must be in [1, 65535]");
-  }
-  CfLauncher launch = pick_contrib(c->n_angles);
-  BART_REQUIRE(ctx, launch != nullptr, "n_angles must be 1, 2, 4, 8 or 16");
-  BART_REQUIRE(ctx, g->n_species <= 4, "contribution functions support 1-4 species");
-  const int S = g->n_species, L = g->n_layers, M = g->n_temps, n = b->n;
-  const int64_t N = g->nu.n_nu;
-  BART_REQUIRE(ctx, (int64_t)n * L <= 2147483647LL, "n x n_layers too large");
-  BART_CUDA(ctx, cudaSetDevice(ctx->device));
-  EmPrep pr;
-  if ((st = emission_prologue(ctx, g, c, b, &pr)) != BART_OK) return st;
-  float* out = contrib;
-  if (!out) {
-    void* p = nullptr;
-    if ((st = bart_scratch(ctx, "cf_rows", (size_t)n * L * N * sizeof(float), &p)) != BART_OK) return st;
-    out = (float*)p;
-  }
-  const int mode = emission_mode(g, c);
-  const int64_t n_tiles = (N + CF_THREADS - 1) / CF_THREADS;
-  launch(dim3((unsigned)n, (unsigned)n_tiles), ctx->stream, g->grid, S, L, M, N, pr.tw, pr.coef,
-         pr.dc + pr.off_dpg, pr.dc + pr.off_ang, g->nu.nu_start_cm, g->nu.dnu_cm, b->nu_lo, b->nu_hi, out, b->active,
-         ctx->d_status, emission_extra(g, c), mode & 1, (mode >> 1) & 1);
-  if ((st = bart_check_launch(ctx, "contrib_kernel")) != BART_OK) return st;
-  if (nb > 0) {
-    contrib_band_kernel<<<dim3((unsigned)(n * L), (unsigned)nb), 256, 0, ctx->stream>>>(
-        out, L, N, b->nu_lo, b->nu_hi, f->weights, nb, b->active, bands);
-    if ((st = bart_check_launch(ctx, "contrib_band_kernel")) != BART_OK) return st;
-  }
-  return BART_OK;
 }
 
 // ---------------------------------------------------------------------------
