@@ -17,49 +17,16 @@
 // the products are those of BF16 weights with FP32 activations to ~1e-5.  The
 // FP32-weight test mode keeps a SIMT FP32 GEMM (64 x 64 tiles, 4 x 4 outputs
 // per thread), the reference precision of the gradient tests.
-#include <cuda_bf16.h>
-
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
-#include <vector>
 
-#include "bart_internal.cuh"
-
-struct bart_mlp {
-  bart_ctx* ctx = nullptr;
-  std::vector<int> widths;
-  int n_layers = 0;
-  int64_t n_params = 0;
-  int bf16 = 1;
-  int log_outputs = 0;
-  int max_batch = 0;
-  int64_t step = 0;
-  std::vector<int64_t> w_off, b_off;   // offsets into the flat vector
-  float* p = nullptr;                  // master FP32 params
-  float* m = nullptr;                  // Adam moments
-  float* v = nullptr;
-  float* g = nullptr;                  // gradient
-  __nv_bfloat16* wb = nullptr;         // BF16 weights (same offsets as p)
-  float* act = nullptr;                // activations: per layer z and h, [max_batch][width]
-  std::vector<int64_t> z_off, h_off;
-  float* scale = nullptr;              // in_shift[in], in_scale[in], out_shift[out], out_scale[out]
-  float* loss = nullptr;
-  float* part = nullptr;               // K-slice partial sums of the tensor-core GEMMs
-  int64_t part_elems = 0;
-  float* xg = nullptr;                 // gathered batch inputs [max_batch][in] (bart_mlp_train_steps)
-  float* tg = nullptr;                 // gathered batch targets [max_batch][out]
-};
+#include "mlp.cuh"
 
 namespace {
 
 constexpr int TM = 64, TN = 64, TK = 16;   // CTA tile and K step
 constexpr int MLP_THREADS = 256;           // 16 x 16 threads, 4 x 4 outputs each
-
-__device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.3989422804014327f * expf(-0.5f * x * x);
-}
 
 template <typename T>
 __device__ __forceinline__ float ld(const T* p) { return (float)p[0]; }
@@ -132,10 +99,6 @@ gemm_kernel(int M, int N, int K, const TA* __restrict__ A, int64_t sam, int64_t 
 }
 
 // ---- BF16 splitting of the tensor-core operands
-__device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-  hi = __float2bfloat16_rn(v);
-  lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
 __device__ __forceinline__ void split_bf16(__nv_bfloat16 v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
   hi = v;
   lo = __float2bfloat16_rn(0.0f);
@@ -191,20 +154,6 @@ __device__ __forceinline__ unsigned int um_smem_u32(const void* p) {
   return (unsigned int)__cvta_generic_to_shared(p);
 }
 
-// Shared-memory matrix descriptor of tcgen05: start address, leading- and
-// stride-dimension byte offsets (all >> 4), the fixed version bits 46..48 =
-// 0b001, no swizzle.
-__device__ __forceinline__ unsigned long long um_desc(unsigned int addr, unsigned int lbo, unsigned int sbo) {
-  return (unsigned long long)((addr & 0x3FFFFu) >> 4) | ((unsigned long long)(lbo >> 4) << 16) |
-         ((unsigned long long)(sbo >> 4) << 32) | (1ull << 46);
-}
-
-// Instruction descriptor of tcgen05.mma kind::f16: FP32 accumulator, BF16 A
-// and B, both K-major, N >> 3 at bits 17..22, M >> 4 at bits 24..28.
-__host__ __device__ constexpr unsigned int um_idesc(int m, int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned int)(n >> 3) << 17) | ((unsigned int)(m >> 4) << 24);
-}
-
 __device__ __forceinline__ bool um_wait(unsigned long long* bar, unsigned int parity) {
   const unsigned int a = um_smem_u32(bar);
   for (unsigned int it = 0; it < UM_SPIN_LIMIT; ++it) {
@@ -217,17 +166,6 @@ __device__ __forceinline__ bool um_wait(unsigned long long* bar, unsigned int pa
     if (ok) return true;
   }
   return false;
-}
-
-// D (+)= A B^T for one 128 x N x 16 step: A and B from their descriptors, D
-// in tensor memory; acc = 0 overwrites D
-__device__ __forceinline__ void um_mma(unsigned int tmem, unsigned long long a, unsigned long long b,
-                                       unsigned int idesc, unsigned int acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
 }
 
 // byte offset of element (r, k) of a [rows][UM_BK] operand tile
@@ -696,13 +634,18 @@ extern "C" bart_status bart_mlp_create(bart_ctx* ctx, const int32_t* widths, int
     amax = std::max<int64_t>(amax, (int64_t)max_batch * std::max(widths[l], widths[l + 1]));
   }
   net->part_elems = std::max(16 * wmax, 16 * amax);
+  net->fused = net->bf16 && n_widths - 1 <= MF_MAX_LAYERS;
+  for (int i = 0; i < n_widths; ++i) net->fused = net->fused && widths[i] <= MF_WIDTH;
   bool ok = cudaMalloc(&net->p, o * 4) == cudaSuccess && cudaMalloc(&net->m, o * 4) == cudaSuccess &&
             cudaMalloc(&net->v, o * 4) == cudaSuccess && cudaMalloc(&net->g, o * 4) == cudaSuccess &&
-            cudaMalloc(&net->wb, o * 2) == cudaSuccess && cudaMalloc(&net->act, a * 4) == cudaSuccess &&
-            cudaMalloc(&net->scale, n_scale * 4) == cudaSuccess && cudaMalloc(&net->loss, 4) == cudaSuccess &&
-            cudaMalloc(&net->part, (size_t)net->part_elems * 4) == cudaSuccess &&
-            cudaMalloc(&net->xg, (size_t)max_batch * widths[0] * 4) == cudaSuccess &&
-            cudaMalloc(&net->tg, (size_t)max_batch * widths[n_widths - 1] * 4) == cudaSuccess;
+            cudaMalloc(&net->scale, n_scale * 4) == cudaSuccess && cudaMalloc(&net->loss, 4) == cudaSuccess;
+  if (net->fused)
+    ok = ok && mlp_fused_create(net);
+  else
+    ok = ok && cudaMalloc(&net->wb, o * 2) == cudaSuccess && cudaMalloc(&net->act, a * 4) == cudaSuccess &&
+         cudaMalloc(&net->part, (size_t)net->part_elems * 4) == cudaSuccess &&
+         cudaMalloc(&net->xg, (size_t)max_batch * widths[0] * 4) == cudaSuccess &&
+         cudaMalloc(&net->tg, (size_t)max_batch * widths[n_widths - 1] * 4) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     bart_mlp_destroy(net);
@@ -715,7 +658,8 @@ extern "C" bart_status bart_mlp_create(bart_ctx* ctx, const int32_t* widths, int
   BART_CUDA(ctx, cudaMemset(net->p, 0, o * 4));
   BART_CUDA(ctx, cudaMemset(net->m, 0, o * 4));
   BART_CUDA(ctx, cudaMemset(net->v, 0, o * 4));
-  BART_CUDA(ctx, cudaMemset(net->wb, 0, o * 2));
+  if (net->fused) BART_CUDA(ctx, cudaMemset(net->pack, 0, net->pack_bytes));
+  else BART_CUDA(ctx, cudaMemset(net->wb, 0, o * 2));
   *out = net;
   return BART_OK;
 }
@@ -725,7 +669,8 @@ extern "C" void bart_mlp_destroy(bart_mlp* net) {
   cudaSetDevice(net->ctx->device);
   cudaStreamSynchronize(net->ctx->stream);
   for (void* q : {(void*)net->p, (void*)net->m, (void*)net->v, (void*)net->g, (void*)net->wb, (void*)net->act,
-                  (void*)net->scale, (void*)net->loss, (void*)net->part, (void*)net->xg, (void*)net->tg})
+                  (void*)net->scale, (void*)net->loss, (void*)net->part, (void*)net->xg, (void*)net->tg,
+                  (void*)net->pack, (void*)net->tr, (void*)net->gpart, (void*)net->bpart, (void*)net->lpart})
     if (q) cudaFree(q);
   delete net;
 }
@@ -756,8 +701,9 @@ extern "C" bart_status bart_mlp_set_params(bart_mlp* net, const float* params) {
   BART_CUDA(net->ctx, cudaMemcpyAsync(net->p, params, net->n_params * 4, cudaMemcpyDeviceToDevice, st));
   BART_CUDA(net->ctx, cudaMemsetAsync(net->m, 0, net->n_params * 4, st));
   BART_CUDA(net->ctx, cudaMemsetAsync(net->v, 0, net->n_params * 4, st));
-  to_bf16<<<blocks_for(net->n_params, 256), 256, 0, st>>>(net->p, net->wb, net->n_params);
   net->step = 0;
+  if (net->fused) return mlp_fused_pack(net);
+  to_bf16<<<blocks_for(net->n_params, 256), 256, 0, st>>>(net->p, net->wb, net->n_params);
   return bart_check_launch(net->ctx, "to_bf16");
 }
 
@@ -774,6 +720,7 @@ extern "C" bart_status bart_mlp_forward(bart_mlp* net, const float* x, int B, fl
   BART_REQUIRE(net->ctx, x && y, "NULL x or y");
   bart_status st = check_batch(net, B);
   if (st != BART_OK) return st;
+  if (net->fused) return mlp_fused_forward(net, x, B, y);
   const int ni = net->widths[0], no = net->widths[net->n_layers];
   cudaStream_t s = net->ctx->stream;
   scale_inputs<<<blocks_for((int64_t)B * ni, 256), 256, 0, s>>>(x, B, ni, net->scale, net->scale + ni,
@@ -791,6 +738,7 @@ extern "C" bart_status bart_mlp_gradient(bart_mlp* net, const float* x, const fl
   BART_REQUIRE(net->ctx, x && t, "NULL x or t");
   bart_status st = check_batch(net, B);
   if (st != BART_OK) return st;
+  if (net->fused) return mlp_fused_gradient(net, x, t, B, nullptr, B, grad, loss, nullptr);
   if ((st = backward(net, x, t, B, loss)) != BART_OK) return st;
   if (grad)
     BART_CUDA(net->ctx, cudaMemcpyAsync(grad, net->g, net->n_params * 4, cudaMemcpyDeviceToDevice,
@@ -800,14 +748,32 @@ extern "C" bart_status bart_mlp_gradient(bart_mlp* net, const float* x, const fl
 
 namespace {
 
-// One Adam step on the batch (x, t): gradient, moments, BF16 copy.
-bart_status adam_step(bart_mlp* net, const float* x, const float* t, int B, float lr, float* loss) {
+// One Adam step on the batch (x, t) (rows of the n_rows rows, or rows 0 ..
+// B-1 where rows is NULL): gradient, moments, BF16 copy.
+bart_status adam_step(bart_mlp* net, const float* x, const float* t, int64_t n_rows, const int32_t* rows, int B,
+                      float lr, float* loss) {
   bart_status st;
+  const float c1 = (float)(1.0 - std::pow(0.9, (double)(net->step + 1)));
+  const float c2 = (float)(1.0 - std::pow(0.999, (double)(net->step + 1)));
+  if (net->fused) {
+    const MlpAdam adam{lr, c1, c2};
+    if ((st = mlp_fused_gradient(net, x, t, n_rows, rows, B, nullptr, loss, &adam)) != BART_OK) return st;
+    net->step += 1;
+    return BART_OK;
+  }
+  if (rows) {
+    const int ni = net->widths[0], no = net->widths[net->n_layers];
+    cudaStream_t s = net->ctx->stream;
+    gather_rows<<<blocks_for((int64_t)B * ni, 256), 256, 0, s>>>(x, n_rows, ni, rows, B, net->xg,
+                                                                 net->ctx->d_status);
+    gather_rows<<<blocks_for((int64_t)B * no, 256), 256, 0, s>>>(t, n_rows, no, rows, B, net->tg,
+                                                                 net->ctx->d_status);
+    x = net->xg;
+    t = net->tg;
+  }
   if ((st = backward(net, x, t, B, loss)) != BART_OK) return st;
   net->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = (float)(1.0 - std::pow(0.9, (double)net->step));
-  const float c2 = (float)(1.0 - std::pow(0.999, (double)net->step));
   cudaStream_t s = net->ctx->stream;
   adam_kernel<<<blocks_for(net->n_params, 256), 256, 0, s>>>(net->p, net->m, net->v, net->g, net->n_params, lr, b1,
                                                             b2, 1e-8f, c1, c2);
@@ -824,7 +790,7 @@ extern "C" bart_status bart_mlp_train_step(bart_mlp* net, const float* x, const 
   BART_REQUIRE(net->ctx, lr > 0 && std::isfinite(lr), "lr must be > 0");
   bart_status st = check_batch(net, B);
   if (st != BART_OK) return st;
-  return adam_step(net, x, t, B, lr, loss);
+  return adam_step(net, x, t, B, nullptr, B, lr, loss);
 }
 
 extern "C" bart_status bart_mlp_train_steps(bart_mlp* net, const float* x, const float* t, int64_t n_rows,
@@ -837,15 +803,8 @@ extern "C" bart_status bart_mlp_train_steps(bart_mlp* net, const float* x, const
   if (st != BART_OK) return st;
   for (int k = 0; k < n_steps; ++k)
     BART_REQUIRE(net->ctx, lr[k] > 0 && std::isfinite(lr[k]), "lr[%d] must be > 0", k);
-  const int ni = net->widths[0], no = net->widths[net->n_layers];
-  cudaStream_t s = net->ctx->stream;
-  for (int k = 0; k < n_steps; ++k) {
-    const int32_t* rows = batch_rows + (int64_t)k * B;
-    gather_rows<<<blocks_for((int64_t)B * ni, 256), 256, 0, s>>>(x, n_rows, ni, rows, B, net->xg,
-                                                                 net->ctx->d_status);
-    gather_rows<<<blocks_for((int64_t)B * no, 256), 256, 0, s>>>(t, n_rows, no, rows, B, net->tg,
-                                                                 net->ctx->d_status);
-    if ((st = adam_step(net, net->xg, net->tg, B, lr[k], loss ? loss + k : nullptr)) != BART_OK) return st;
-  }
+  for (int k = 0; k < n_steps; ++k)
+    if ((st = adam_step(net, x, t, n_rows, batch_rows + (int64_t)k * B, B, lr[k], loss ? loss + k : nullptr)) != BART_OK)
+      return st;
   return bart_check_launch(net->ctx, "mlp train steps");
 }
