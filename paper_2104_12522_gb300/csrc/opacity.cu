@@ -48,8 +48,9 @@
 #include <cmath>
 #include <cstddef>
 
-#include "bart_internal.cuh"
-#include "faddeeva.cuh"
+#include "opacity.cuh"
+
+using namespace bartop;
 
 namespace {
 
@@ -60,44 +61,6 @@ constexpr int OP_R_LOG = 4;
 constexpr int OP_SPAN = 32 * OP_R;               // points per warp
 constexpr int OP_TILE = OP_WARPS * OP_SPAN;      // points per CTA
 constexpr float CORE_S = 576.0f;                 // |z|^2 of the core boundary
-constexpr float LN_SCALE = 69.314718055994531f;   // ln(2^100): internal scale of all terms
-constexpr float INV_SCALE = 7.888609052210118e-31f; // 2^-100
-constexpr float LOG2EF = 1.4426950408889634f;
-constexpr float LN2F_ = 0.6931471805599453f;
-
-__device__ __forceinline__ float ex2f_approx(float a) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-__device__ __forceinline__ float lg2f_approx(float a) {
-  float r;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-
-struct LineWin {            // per line, from the FP64 prologue
-  int jlo, jhi, jc;
-  float delta;              // nu_jc - nu0 (cm^-1)
-  float ln_s0;              // ln S_ref + c2 E''/T_ref - ln(1 - exp(-c2 nu0/T_ref)): the T-free part of ln S(T)
-  float c2e;                // c2 E''
-  float c2nu;               // c2 nu0
-  float nu0f;               // nu0 in FP32
-};
-
-struct CellConst {
-  float inv_t;              // 1 / T
-  float ln_q;               // 1.5 ln(296 / T): partition-function ratio
-  float gfac;               // P sqrt(296 / T)  (bar)
-  float dfac;               // sqrt(2 k T / m) / c: sigma*sqrt2 = nu0 * dfac
-  float c2_t;               // c2 / T
-};
-
-__device__ __forceinline__ double nu_minus(double nu_start, double dnu, int64_t j, double nu0) {
-  // (nu_start + j*dnu) - nu0, each operation rounded separately (no FMA).
-  return __dadd_rn(__dadd_rn(nu_start, __dmul_rn((double)j, dnu)), -nu0);
-}
-
 __global__ void line_window_kernel(const double* __restrict__ nu0, const float* __restrict__ log_s,
                                    const float* __restrict__ elow, int64_t n_lines, double nu_start,
                                    double dnu, int64_t n_nu, double cutoff, int* __restrict__ jlo,
@@ -138,20 +101,6 @@ __global__ void line_window_kernel(const double* __restrict__ nu0, const float* 
   win[i] = w;
 }
 
-// ln S(T) = ln_s0 + 1.5 ln(T_ref/T) - c2 E''/T + ln(1 - exp(-c2 nu0/T)), in FP32
-// (the staging of the opacity kernel and the threshold prologue share it).
-__device__ __forceinline__ float line_ln_s(const LineWin& w, const CellConst& cc) {
-  const float stim = 1.0f - ex2f_approx(-w.c2nu * cc.inv_t * LOG2EF);
-  return w.ln_s0 + cc.ln_q - w.c2e * cc.inv_t + LN2F_ * lg2f_approx(stim);
-}
-
-// Order-preserving map of floats to ints (for atomicMax on floats).
-__device__ __forceinline__ int ordered_int(float f) {
-  const int i = __float_as_int(f);
-  return i >= 0 ? i : i ^ 0x7fffffff;
-}
-__device__ __forceinline__ float ordered_float(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
-
 // Largest ln S(T) of a species' lines at each temperature (Sec. 4 item 6:
 // the line-strength bound is relative to the strongest line at each cell; S
 // depends on T only).  smax[blockIdx.y] must start at a very negative
@@ -173,15 +122,6 @@ __global__ void line_smax_kernel(const LineWin* __restrict__ win, int64_t n_line
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (threadIdx.x == 0) atomicMax(&smax[blockIdx.y], ordered_int(m));
   }
-}
-
-// First index in [lo, hi) with key[i] >= v (key nondecreasing).
-__device__ int64_t lower_bound_i(const int* __restrict__ key, int64_t lo, int64_t hi, int v) {
-  while (lo < hi) {
-    int64_t mid = (lo + hi) >> 1;
-    if (key[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
 }
 
 // Line ranges of one warp span [w0, w0 + OP_SPAN - 1] (independent of the
@@ -416,7 +356,8 @@ __global__ void __launch_bounds__(OP_THREADS, 3)
 opacity_kernel(const LineWin* __restrict__ win, const float* __restrict__ gref,
                const SpanRange* __restrict__ spans, const CellConst* __restrict__ cells, double dnu,
                int64_t n_nu, float* __restrict__ out, const float2* __restrict__ wtab,
-               const int* __restrict__ smax, const int* __restrict__ tmap, float ln_rel) {
+               const int* __restrict__ smax, const int* __restrict__ tmap, float ln_rel,
+               const DensePlan* __restrict__ plan) {
   extern __shared__ __align__(16) unsigned char op_smem[];
   OpShared& sh = *reinterpret_cast<OpShared*>(op_smem);
 
@@ -427,6 +368,7 @@ opacity_kernel(const LineWin* __restrict__ win, const float* __restrict__ gref,
   const int j0 = w0 + lane * OP_R;          // first point of this lane
   const float j0r = (float)(lane * OP_R);   // its offset in the span
   const int cell = blockIdx.y;
+  if (plan && plan[cell].m1) return;        // written by the kernels for dense lists
   const CellConst cc = cells[cell];
   // line-strength bound: lines with ln S below this are left out
   const float ln_thr = smax ? ordered_float(smax[tmap[cell]]) + ln_rel : -3.0e38f;
@@ -889,7 +831,7 @@ bart_status run_cells(bart_ctx* ctx, const bart_linelist* species, int n_species
   for (int s = 0; s < n_species; ++s)
     for (int c = 0; c < n_cells; ++c) {
       const double T = t[c], P = p[c];
-      CellConst k;
+      CellConst k{};
       k.inv_t = (float)(1.0 / T);
       k.ln_q = (float)(1.5 * std::log(bartc::TREF / T));
       k.gfac = (float)(P * std::sqrt(bartc::TREF / T));
@@ -897,6 +839,9 @@ bart_status run_cells(bart_ctx* ctx, const bart_linelist* species, int n_species
       k.c2_t = (float)(bartc::C2 / T);
       hc[(size_t)s * n_cells + c] = k;
     }
+  std::vector<char> dense(n_species);      // species with cells on the kernels for dense lists
+  for (int s = 0; s < n_species; ++s)
+    dense[s] = dense_applies(species[s], nu, cutoff, hc.data() + (size_t)s * n_cells, n_cells);
   if ((st = bart_upload_const(ctx, "op_cells", hc.data(), hc.size() * sizeof(CellConst), &p_cells)) != BART_OK)
     return st;
   BART_CUDA(ctx, cudaFuncSetAttribute(opacity_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -951,11 +896,17 @@ bart_status run_cells(bart_ctx* ctx, const bart_linelist* species, int n_species
         if ((st = bart_check_launch(ctx, "line_smax_kernel")) != BART_OK) return st;
       }
     }
+    const DensePlan* plan = nullptr;
+    if (dense[s] &&
+        (st = dense_cells(ctx, (const LineWin*)p_win, (const int*)p_jlo, (const int*)p_jhi, L.gamma_ref_cm, L.n_lines,
+                          (const CellConst*)p_cells + (size_t)s * n_cells, n_cells, nu, cutoff,
+                          thr ? (const int*)p_smax : nullptr, (const int*)p_tmap, ln_rel, o, &plan)) != BART_OK)
+      return st;
     dim3 grid((unsigned)n_tiles, (unsigned)n_cells);
     opacity_kernel<<<grid, OP_THREADS, sizeof(OpShared), ctx->stream>>>(
         (const LineWin*)p_win, L.gamma_ref_cm, (const SpanRange*)p_spans,
         (const CellConst*)p_cells + (size_t)s * n_cells, nu.dnu_cm, nu.n_nu, o, ctx->d_wtable,
-        thr ? (const int*)p_smax : nullptr, (const int*)p_tmap, ln_rel);
+        thr ? (const int*)p_smax : nullptr, (const int*)p_tmap, ln_rel, plan);
     if ((st = bart_check_launch(ctx, "opacity_kernel")) != BART_OK) return st;
   }
   return BART_OK;
@@ -1157,7 +1108,7 @@ bart_status run_cells_table(bart_ctx* ctx, const bart_voigt_table* tab, const ba
   for (int s = 0; s < n_species; ++s)
     for (int c = 0; c < n_cells; ++c) {
       const double T = t[c], P = p[c];
-      CellConst k;
+      CellConst k{};
       k.inv_t = (float)(1.0 / T);
       k.ln_q = (float)(1.5 * std::log(bartc::TREF / T));
       k.gfac = (float)(P * std::sqrt(bartc::TREF / T));
