@@ -368,7 +368,7 @@ opacity_kernel(const LineWin* __restrict__ win, const float* __restrict__ gref,
   const int j0 = w0 + lane * OP_R;          // first point of this lane
   const float j0r = (float)(lane * OP_R);   // its offset in the span
   const int cell = blockIdx.y;
-  if (plan && plan[cell].m1) return;        // written by the kernels for dense lists
+  if (plan && plan[cell].kind != DN_NONE) return;        // written by the kernels for dense lists
   const CellConst cc = cells[cell];
   // line-strength bound: lines with ln S below this are left out
   const float ln_thr = smax ? ordered_float(smax[tmap[cell]]) + ln_rel : -3.0e38f;

@@ -72,11 +72,13 @@ __device__ inline int64_t lower_bound_i(const int* __restrict__ key, int64_t lo,
   return lo;
 }
 
-// Per (P, T) cell: near radius in blocks of 8 points and far radius in blocks
-// of 32 points of the kernels for dense lists; m1 = 0: the cell is computed
-// line by line (opacity_kernel).
+// Per (P, T) cell, what the kernels for dense lists do (opacity_dense.cu): near
+// radius m1 in blocks of 8 points; blocks of 32 points from m2 blocks on by
+// their moments about the centre, from mh on by those about complex centres
+// (DN_COMPLEX).
+enum { DN_NONE = 0, DN_REAL = 1, DN_COMPLEX = 2 };   // DN_NONE: line by line (opacity_kernel)
 struct DensePlan {
-  int m1, m2;
+  int kind, m1, mh, m2;
 };
 
 // Whether a species' list is dense enough on this grid for those kernels;

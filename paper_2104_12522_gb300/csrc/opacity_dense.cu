@@ -24,6 +24,15 @@
 // first term left out is then below 9 DN_RHO^8 = 1.3e-6 of a line's own at the
 // nearest point for the line farthest from the centre, far below that in a sum.
 //
+// Lorentz widths beyond about 3 points need moments about a complex centre:
+// with the lines of a block in bins of gamma_ref (ratio <= sqrt 2 within a bin),
+// u = delta + g + i (gamma - gamma_c) about the bin's middle gamma_c and
+// Z = d - i gamma_c, V = (S / pi) Im sum_n E[u^n] / Z^(n+1): |Z| >= gamma_c, so a
+// wide profile is smooth on the scale of a block and needs no near lines at
+// all.  DN_PC terms hold where |u| <= DN_RHOC |Z| (15 DN_RHOC^14 = 9e-7).
+// Distances where the moments about the real centre hold take those (one set
+// per block, half the operations).
+//
 // Near lines.  A warp takes one source block, a lane one line: constants,
 // moments and all the block's near points (8 (2 m1 - 1), the same for all lanes)
 // without a line's constants leaving its registers, so lanes agree on how far
@@ -36,13 +45,18 @@
 // blocks around a point, then the moments.  No atomics: every sum has a fixed
 // order.
 //
-// Used (dense_applies, plan_kernel) for lists of at least DN_DENSITY lines per
-// point, where blocks pay for their fixed cost, and for cells whose widths fit:
-// Doppler widths that keep |x| >= 9 from the first mid block on, Lorentz widths
-// up to about 3 grid points (m1 <= DN_M1_MAX).  Other cells go line by line.
+// Used (dense_applies, dense_plan_kernel) for lists of at least DN_DENSITY lines
+// per point, where blocks pay for their fixed cost, and for cells whose widths
+// fit: Doppler widths that keep |x| >= 9 from the first mid block on; Lorentz
+// widths up to about 3 grid points, or gamma_ref within a factor 4 over the
+// list (4 bins) and widths below a sixth of the cutoff (the moments of the
+// divided blocks are about the real centre), or a cutoff so short that the near
+// window holds all of it.  Other cells go line by line.
 // Measured: one species of the 5e6-line grid (1.67e6 lines, 100,000 points), 10
 // layers over 1e-8 .. 100 bar x 20 temperatures: 169 ms line by line, 58 ms with
-// 160 of the 200 cells here.
+// the 160 cells of widths up to 3 points here, 44 ms with the wider ones too;
+// 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart: 2.59 ms and
+// 0.33 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -58,11 +72,16 @@ constexpr int DN_M1 = 4, DN_M1_MAX = 5;     // near radius in blocks
 constexpr int DN_WIN = (2 * DN_M1_MAX - 1) * DN_B;   // near points of a block, at most
 constexpr int DN_GROUPS = 20;               // groups of a block: jlo and jhi each step at most 9 times
 constexpr float DN_RHO = 0.14f;
+constexpr int DN_BINS = 4;                  // bins of gamma_ref
+constexpr int DN_PC = 14;                   // moments about a complex centre
+constexpr float DN_RHOC = 0.305f;
+constexpr float DN_RHO_EDGE = 0.175f;       // divided blocks: 9 x 0.175^8 = 8e-6 of a line at its cutoff
 constexpr double DN_DENSITY = 0.5;          // lines per point
 constexpr int DN_WARPS = 4;
 constexpr int DN_FOLD = 8;                  // chunks of 32 lines between two folds
 constexpr float DN_EPS_L = 2e-6f;           // bound of the shifted Lorentz form
-constexpr size_t DN_SCRATCH = (size_t)96 << 20;      // moments and windows of a batch of cells: within L2
+constexpr size_t DN_SCRATCH = (size_t)256 << 20;     // moments and windows of a batch of cells (a third of it is
+                                                     // touched for a cell: within L2)
 
 struct DensePoint {           // per grid point (indexes of groups and blocks)
   int gl, gr;                 // groups whose window holds the point: [gl, gr)
@@ -183,36 +202,81 @@ __global__ void dense_point_kernel(const LineWin* __restrict__ win, const int* _
 }
 
 // stat[0]: largest gamma_ref (bits of a non-negative float), stat[1]: a value
-// that is negative or not a number.
+// that is negative or not a number, stat[2]: 0x7fffffff - bits of the smallest.
 __global__ void __launch_bounds__(256)
 dense_gamma_kernel(const float* __restrict__ gref, int64_t n, int* __restrict__ stat) {
-  unsigned m = 0;
+  unsigned m = 0, mi = 0;
   bool bad = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float g = gref[i];
     bad |= !(g >= 0.0f);
-    m = max(m, __float_as_uint(fmaxf(g, 0.0f)));
+    const unsigned bits = __float_as_uint(fmaxf(g, 0.0f)) & 0x7fffffffu;
+    m = max(m, bits);
+    mi = max(mi, 0x7fffffffu - bits);
   }
   m = __reduce_max_sync(0xffffffffu, m);
+  mi = __reduce_max_sync(0xffffffffu, mi);
   bad = __any_sync(0xffffffffu, bad);
   if ((threadIdx.x & 31) == 0) {
     if (m) atomicMax(stat, (int)m);
+    if (mi) atomicMax(stat + 2, (int)mi);
     if (bad) atomicOr(stat + 1, 1);
   }
 }
 
+// Bins of gamma_ref: n of equal ratio over the list's range, 0 if it does not
+// fit; middle and reach of the bins, at 1 bar and 296 K.
+struct DenseBins {
+  int n;
+  float inv_g0, inv_lr;       // bin of g: floor(log2(g inv_g0) inv_lr)
+  float eta;                  // half width of a bin over its middle
+  float c[DN_BINS];
+};
+
+__device__ DenseBins dense_bins(const int* __restrict__ stat) {
+  DenseBins r{};
+  const float g1 = __int_as_float(stat[0]), g0 = __int_as_float(0x7fffffff - stat[2]);
+  if (!(g0 > 1e-30f) || !(g1 < 1e30f)) return r;
+  const float lr = log2f(g1 / g0);
+  const int n = max(1, (int)ceilf(2.0f * lr - 1e-3f));
+  if (n > DN_BINS) return r;
+  r.n = n;
+  r.inv_g0 = 1.0f / g0;
+  r.inv_lr = lr > 0.0f ? (float)n / lr : 0.0f;
+  const float rb = exp2f(lr / n);
+  r.eta = (rb - 1.0f) / (rb + 1.0f);
+  for (int q = 0; q < n; ++q) r.c[q] = g0 * exp2f(lr * q / n) * 0.5f * (1.0f + rb);
+  return r;
+}
+
 __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cells, const int* __restrict__ stat,
-                                  float inv_dnu, DensePlan* __restrict__ plan) {
+                                  float inv_dnu, int reach, DensePlan* __restrict__ plan,
+                                  DenseBins* __restrict__ bins) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const DenseBins bn = dense_bins(stat);
+  if (c == 0) *bins = bn;
   if (c >= n_cells) return;
-  DensePlan p{0, 0};
-  const float g = __int_as_float(stat[0]) * cells[c].gfac * inv_dnu;   // largest Lorentz width, in points
+  DensePlan p{DN_NONE, 0, 0, 0};
+  const float scale = cells[c].gfac * inv_dnu, g = __int_as_float(stat[0]) * scale;   // widest line, in points
   if (cells[c].dense && !stat[1] && g < 1e6f) {
     // a point of block t is at least 8 m - 3.5 points from the centre of block t +- m
     const int m1 = max(DN_M1, (int)ceilf((sqrtf(16.0f + g * g) / DN_RHO + 3.5f) / 8.0f));
+    const int m2 = max(4, (int)ceilf((sqrtf(256.0f + g * g) / DN_RHO + 15.5f) / 32.0f));
     if (m1 <= DN_M1_MAX) {
-      p.m1 = m1;
-      p.m2 = max(4, (int)ceilf((sqrtf(256.0f + g * g) / DN_RHO + 15.5f) / 32.0f));
+      p = {DN_REAL, m1, 0, m2};
+    } else if (8 * (DN_M1_MAX - 1) > reach) {    // the near window holds every line's points
+      p = {DN_REAL, DN_M1_MAX, 0, m2};
+    } else if (bn.n > 0 && sqrtf(16.0f + g * g) <= DN_RHO_EDGE * (float)(reach - 8)) {
+      float d8 = 0.0f, d32 = 0.0f;               // squared distances from which the complex moments hold
+      for (int q = 0; q < bn.n; ++q) {
+        const float gc = bn.c[q] * scale, e2 = bn.eta * bn.eta * gc * gc;
+        d8 = fmaxf(d8, (16.0f + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
+        d32 = fmaxf(d32, (256.0f + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
+      }
+      p.kind = DN_COMPLEX;
+      p.m1 = d8 > 0.0f ? (int)ceilf((sqrtf(d8) + 3.5f) / 8.0f) : 0;
+      p.mh = d32 > 0.0f ? (int)ceilf((sqrtf(d32) + 15.5f) / 32.0f) : 0;
+      p.m2 = max(m2, p.mh);
     }
   }
   plan[c] = p;
@@ -305,6 +369,7 @@ struct DenseArgs {
   const CellConst* cells;
   const DensePlan* plan;
   const DensePoint* pts;
+  const DenseBins* bins;
   const int* smax;
   const int* tmap;
   const float2* wtab;
@@ -315,6 +380,8 @@ struct DenseArgs {
   float* m8;                                 // [cell][nb][DN_P]
   float* m32;                                // [cell][nb / 4][DN_P]
   float* mg;                                 // [cell][g_stride][DN_P]
+  float2* mc8;                               // [cell][nb][DN_BINS][DN_PC], complex centres
+  float2* mc32;                              // [cell][nb / 4][DN_BINS][DN_PC]
   float* out;
 };
 
@@ -331,16 +398,17 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
   const int b = blockIdx.x * DN_WARPS + warp;
   const int cell = a.c0 + blockIdx.y;
   const DensePlan plan = a.plan[cell];
-  if (plan.m1 == 0 || b >= a.nb) return;     // warps are independent: no CTA barrier below
+  if (plan.kind == DN_NONE || b >= a.nb) return;   // warps are independent: no CTA barrier below
   const int l0 = a.lstart[b], l1 = a.lstart[b + 1];
   // (the bounds hold for any list; a sorted one has no block with more groups)
   const int g0 = a.gfirst[b], ng = max(0, min(min(a.gfirst[b + 1] - g0, DN_GROUPS), (int)a.g_stride - g0));
   const CellConst cc = a.cells[cell];
   const float ln_thr = a.smax ? ordered_float(a.smax[a.tmap[cell]]) + a.ln_rel : -3.0e38f;
-  const int n_pts = (2 * plan.m1 - 1) * DN_B, steps = n_pts / 4;
-  const int w0 = (b - a.boff - (plan.m1 - 1)) * DN_B;         // grid index of the window's first point
-  const float centre = (float)((plan.m1 - 1) * DN_B) + 3.5f;  // the block's centre in the window
-  const bool check = 8 * plan.m1 >= a.reach;                  // the window passes the cutoff
+  const int m1 = max(plan.m1, 1);
+  const int n_pts = plan.m1 > 0 ? (2 * m1 - 1) * DN_B : 0, steps = n_pts / 4;
+  const int w0 = (b - a.boff - (m1 - 1)) * DN_B;              // grid index of the window's first point
+  const float centre = (float)((m1 - 1) * DN_B) + 3.5f;       // the block's centre in the window
+  const bool check = 8 * m1 >= a.reach;                       // the window passes the cutoff
   float4 (*acc)[32] = sh.acc[warp];
   float (*grp)[DN_P] = sh.group[warp];
   for (int s = 0; s < steps; ++s) acc[s][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -494,6 +562,50 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     for (int g = 0; g < ng; ++g) t += grp[g][lane];
     a.m8[at * DN_P + lane] = t;
   }
+  if (plan.kind != DN_COMPLEX) return;
+  // ---- moments about the complex centres, a pass over the lines per bin
+  const DenseBins bn = *a.bins;
+  for (int bin = 0; bin < bn.n; ++bin) {
+    float2 M[DN_PC];
+#pragma unroll
+    for (int n = 0; n < DN_PC; ++n) M[n] = make_float2(0.f, 0.f);
+    const float gc = bn.c[bin] * cc.gfac;
+    for (int base = l0; base < l1; base += 32) {
+      const int i = min(base + lane, l1 - 1);
+      const LineWin w = a.win[i];
+      const float gr = a.gref[i];
+      const int mine = min(max((int)floorf(log2f(gr * bn.inv_g0) * bn.inv_lr), 0), bn.n - 1);
+      const float ln_s = line_ln_s(w, cc);
+      const bool take = base + lane < l1 && mine == bin && ln_s >= ln_thr;
+      const float wt = take ? ex2f_approx((ln_s + LN_SCALE) * LOG2EF) * a.w_scale : 0.0f;
+      const float inv = bartw::rcp_approx(w.nu0f * cc.dfac), rdx = bartw::rcp_approx(a.dnu * inv), s2 = 0.5f * rdx * rdx;
+      const float de = ((float)(w.jc - w0) - centre) - w.delta * a.inv_dnu, ga = (gr * cc.gfac - gc) * a.inv_dnu;
+      // K_0 = 1, K_1 = u, K_(n+1) = u K_n + n sigma^2 K_(n-1), weighted
+      float r0 = wt, i0 = 0.0f, r1 = de * wt, i1 = ga * wt;
+#pragma unroll
+      for (int n = 0; n < DN_PC; ++n) {
+        M[n].x += r0;
+        M[n].y += i0;
+        const float ns = (float)(n + 1) * s2;
+        const float r2 = fmaf(de, r1, fmaf(-ga, i1, ns * r0)), i2 = fmaf(de, i1, fmaf(ga, r1, ns * i0));
+        r0 = r1;
+        i0 = i1;
+        r1 = r2;
+        i1 = i2;
+      }
+    }
+    float2 mine = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int n = 0; n < DN_PC; ++n) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        M[n].x += __shfl_xor_sync(0xffffffffu, M[n].x, o);
+        M[n].y += __shfl_xor_sync(0xffffffffu, M[n].y, o);
+      }
+      if (lane == n) mine = M[n];
+    }
+    if (lane < DN_PC) a.mc8[(at * DN_BINS + bin) * DN_PC + lane] = mine;
+  }
 }
 
 // Moments of the blocks of 32 points from their four blocks of 8: with t the
@@ -501,7 +613,8 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
 __global__ void __launch_bounds__(128)
 dense_up_kernel(const __grid_constant__ DenseArgs a) {
   const int P = blockIdx.x * blockDim.x + threadIdx.x;
-  if (P >= a.nb / 4 || a.plan[a.c0 + blockIdx.y].m1 == 0) return;
+  const int kind = a.plan[a.c0 + blockIdx.y].kind;
+  if (P >= a.nb / 4 || kind == DN_NONE) return;
   const float* m = a.m8 + ((int64_t)blockIdx.y * a.nb + 4 * P) * DN_P;
   float o[DN_P] = {};
 #pragma unroll
@@ -522,6 +635,27 @@ dense_up_kernel(const __grid_constant__ DenseArgs a) {
   float* d = a.m32 + ((int64_t)blockIdx.y * (a.nb / 4) + P) * DN_P;
 #pragma unroll
   for (int n = 0; n < DN_P; ++n) d[n] = o[n];
+  if (kind != DN_COMPLEX) return;
+  for (int bin = 0; bin < a.bins->n; ++bin) {
+    float2 u[DN_PC] = {};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float t = (float)(8 * c - 12);
+      const float2* src = a.mc8 + (((int64_t)blockIdx.y * a.nb + 4 * P + c) * DN_BINS + bin) * DN_PC;
+      float2 v[DN_PC];
+#pragma unroll
+      for (int n = 0; n < DN_PC; ++n) v[n] = src[n];
+#pragma unroll
+      for (int r = 1; r < DN_PC; ++r)
+#pragma unroll
+        for (int n = DN_PC - 1; n >= r; --n) v[n] = make_float2(fmaf(t, v[n - 1].x, v[n].x), fmaf(t, v[n - 1].y, v[n].y));
+#pragma unroll
+      for (int n = 0; n < DN_PC; ++n) u[n] = make_float2(u[n].x + v[n].x, u[n].y + v[n].y);
+    }
+    float2* dst = a.mc32 + (((int64_t)blockIdx.y * (a.nb / 4) + P) * DN_BINS + bin) * DN_PC;
+#pragma unroll
+    for (int n = 0; n < DN_PC; ++n) dst[n] = u[n];
+  }
 }
 
 // sum_n I_n / D^(n+1)
@@ -539,6 +673,24 @@ __device__ __forceinline__ float moment_sum(const float* __restrict__ m, float D
   return v * (r * r);
 }
 
+// Im sum_n M_n / Z^(n+1), Z = D - i g
+__device__ __forceinline__ float complex_sum(const float2* __restrict__ m, float D, float g) {
+  const float q = bartw::rcp_approx(fmaf(D, D, g * g)), rr = D * q, ri = g * q;   // 1 / Z
+  const float4* p = reinterpret_cast<const float4*>(m);
+  float vr = 0.0f, vi = 0.0f;
+#pragma unroll
+  for (int n = DN_PC / 2 - 1; n >= 0; --n) {
+    const float4 c = p[n];                       // M_2n, M_(2n+1)
+    float t = fmaf(vr, rr, fmaf(-vi, ri, c.z));
+    vi = fmaf(vr, ri, fmaf(vi, rr, c.w));
+    vr = t;
+    t = fmaf(vr, rr, fmaf(-vi, ri, c.x));
+    vi = fmaf(vr, ri, fmaf(vi, rr, c.y));
+    vr = t;
+  }
+  return fmaf(vr, ri, vi * rr);
+}
+
 // One point per thread: the warp's 32 points are one block of 32, so its lanes
 // agree on the far blocks and almost on the mid ones (uniform loops, one
 // broadcast read per block).
@@ -546,7 +698,7 @@ __global__ void __launch_bounds__(256)
 dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   const int cell = a.c0 + blockIdx.y;
   const DensePlan plan = a.plan[cell];
-  if (plan.m1 == 0) return;
+  if (plan.kind == DN_NONE) return;
   const int j0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
   if (j0 >= a.n_nu) return;
   const int lane = threadIdx.x & 31, j = min(j0 + lane, a.n_nu - 1);
@@ -569,6 +721,44 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   // ---- blocks inside the point's cutoff [bl, br), outside the near ones
   const int PL = (p.bl + 3) >> 2, PR = p.br >> 2;            // parents inside it
   float far = 0.0f, mid = 0.0f;
+  if (plan.kind == DN_COMPLEX) {
+    const DenseBins bn = *a.bins;
+    const float scale = a.cells[cell].gfac * a.inv_dnu;
+    const float2* mc8 = a.mc8 + (int64_t)blockIdx.y * a.nb * DN_BINS * DN_PC;
+    const float2* mc32 = a.mc32 + (int64_t)blockIdx.y * (a.nb / 4) * DN_BINS * DN_PC;
+    // parents inside the cutoff: real centre far away, complex centres nearer
+    const int u0 = __reduce_min_sync(0xffffffffu, PL), u1 = __reduce_max_sync(0xffffffffu, PR);
+    for (int P = u0; P < u1; ++P) {
+      const int m = abs(P - T);                  // the same for the warp
+      const bool in = P >= PL && P < PR;
+      const float D = jf - centre32(P);
+      if (m >= plan.m2) {
+        if (in) far += moment_sum(m32 + (int64_t)P * DN_P, D);
+      } else if (m >= plan.mh) {
+        for (int q = 0; q < bn.n; ++q)
+          if (in) far += complex_sum(mc32 + ((int64_t)P * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
+      }
+    }
+    // blocks of the parents closer than that, and those beside the parents
+    auto blocks8 = [&](int b0, int b1) {
+      const int v0 = __reduce_min_sync(0xffffffffu, b0 < b1 ? b0 : 0x7fffffff);
+      const int v1 = __reduce_max_sync(0xffffffffu, b0 < b1 ? b1 : -0x7fffffff);
+      for (int b = v0; b < v1; ++b) {
+        const bool in = b >= b0 && b < b1 && abs(b - t) >= plan.m1;
+        const float D = jf - centre8(b);
+        for (int q = 0; q < bn.n; ++q)
+          if (in) mid += complex_sum(mc8 + ((int64_t)b * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
+      }
+    };
+    const int c0 = max(4 * (T - plan.mh + 1), 4 * PL), c1 = min(4 * (T + plan.mh), 4 * PR);
+    if (PL < PR) {
+      blocks8(p.bl, 4 * PL);
+      blocks8(c0, c1);
+      blocks8(4 * PR, p.br);
+    } else {
+      blocks8(p.bl, p.br);
+    }
+  } else {
   // left of the point: parents [PL, PE), blocks before and after them
   const int PE = min(T - plan.m2 + 1, PR), lend = min(t - plan.m1 + 1, p.br);
   const int PS = max(T + plan.m2, PL), rbeg = max(t + plan.m1, p.bl);
@@ -591,6 +781,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   blocks(hasL ? 4 * PE : lend, lend);
   blocks(rbeg, hasR ? 4 * PS : p.br);
   blocks(hasR ? max(4 * PR, rbeg) : p.br, p.br);
+  }
 
   // ---- edges: the block that a cutoff edge divides, group by group (blocks
   // within the near radius were taken line by line)
@@ -644,24 +835,37 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
   const int nb = (boff + n_nu / DN_B + (reach + 2) / DN_B + DN_M1_MAX + 8) / 4 * 4;
   const int tiles = (n + GR_TILE - 1) / GR_TILE;
   const int64_t g_max = std::min<int64_t>(n, (int64_t)nb * DN_GROUPS) + 1;
-  const size_t per_cell = ((size_t)nb * (DN_WIN + DN_P) + (size_t)(nb / 4) * DN_P + (size_t)g_max * DN_P) * 4;
+  const size_t per_cell = ((size_t)nb * (DN_WIN + DN_P) + (size_t)(nb / 4) * DN_P + (size_t)g_max * DN_P +
+                           (size_t)(nb + nb / 4) * DN_BINS * DN_PC * 2) * 4;
   const int batch = (int)std::max<size_t>(1, std::min<size_t>(n_cells, DN_SCRATCH / per_cell));
-  bart_status st;
+  DenseBins* bins;
   int *range, *lstart, *gfirst, *gid, *count, *stat;
   DensePlan* pl;
   DensePoint* pts;
   float* scratch;
-  if ((st = bart_scratch(ctx, "dn_range", 4 * sizeof(int), (void**)&range)) != BART_OK) return st;
-  stat = range + 2;
-  if ((st = bart_scratch(ctx, "dn_lstart", (size_t)(nb + 1) * sizeof(int), (void**)&lstart)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_gfirst", (size_t)(nb + 1) * sizeof(int), (void**)&gfirst)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_gid", (size_t)n * sizeof(int), (void**)&gid)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_count", (size_t)(tiles + 1) * sizeof(int), (void**)&count)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_plan", (size_t)n_cells * sizeof(DensePlan), (void**)&pl)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_pts", (size_t)n_nu * sizeof(DensePoint), (void**)&pts)) != BART_OK) return st;
-  if ((st = bart_scratch(ctx, "dn_moments", per_cell * batch, (void**)&scratch)) != BART_OK) return st;
+  *plan = nullptr;
+  const struct {
+    const char* name;
+    size_t bytes;
+    void** p;
+  } need[] = {{"dn_range", 8 * sizeof(int), (void**)&range},
+              {"dn_bins", sizeof(DenseBins), (void**)&bins},
+              {"dn_lstart", (size_t)(nb + 1) * sizeof(int), (void**)&lstart},
+              {"dn_gfirst", (size_t)(nb + 1) * sizeof(int), (void**)&gfirst},
+              {"dn_gid", (size_t)n * sizeof(int), (void**)&gid},
+              {"dn_count", (size_t)(tiles + 1) * sizeof(int), (void**)&count},
+              {"dn_plan", (size_t)n_cells * sizeof(DensePlan), (void**)&pl},
+              {"dn_pts", (size_t)n_nu * sizeof(DensePoint), (void**)&pts},
+              {"dn_moments", per_cell * batch, (void**)&scratch}};
+  for (const auto& q : need)
+    if (bart_scratch(ctx, q.name, q.bytes, q.p) != BART_OK) {
+      ctx->err.clear();       // no room (or a capture that cannot grow it): every cell goes line by line
+      return BART_OK;
+    }
+  stat = range + 4;
+  bart_status st;
   cudaStream_t s = ctx->stream;
-  BART_CUDA(ctx, cudaMemsetAsync(stat, 0, 2 * sizeof(int), s));
+  BART_CUDA(ctx, cudaMemsetAsync(stat, 0, 3 * sizeof(int), s));
   const int* total = count + tiles;
   dense_range_kernel<<<1, 1, 0, s>>>(jlo, jhi, n, n_nu, range);
   dense_block_kernel<<<nb / 256 + 1, 256, 0, s>>>(win, range, boff, nb, lstart);
@@ -671,7 +875,7 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
   dense_first_group_kernel<<<nb / 256 + 1, 256, 0, s>>>(lstart, range, gid, total, nb, gfirst);
   dense_point_kernel<<<(n_nu + 255) / 256, 256, 0, s>>>(win, jlo, jhi, range, gid, total, lstart, boff, nb, n_nu, pts);
   dense_gamma_kernel<<<std::min(tiles, 4 * ctx->sm_count), 256, 0, s>>>(gref, n, stat);
-  dense_plan_kernel<<<(n_cells + 127) / 128, 128, 0, s>>>(cells, n_cells, stat, (float)(1.0 / nu.dnu_cm), pl);
+  dense_plan_kernel<<<(n_cells + 127) / 128, 128, 0, s>>>(cells, n_cells, stat, (float)(1.0 / nu.dnu_cm), reach, pl, bins);
   if ((st = bart_check_launch(ctx, "dense opacity prologue")) != BART_OK) return st;
   DenseArgs a{};
   a.win = win;
@@ -682,6 +886,7 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
   a.cells = cells;
   a.plan = pl;
   a.pts = pts;
+  a.bins = bins;
   a.smax = smax;
   a.tmap = tmap;
   a.wtab = ctx->d_wtable;
@@ -697,7 +902,9 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
   a.window = scratch;
   a.m8 = a.window + (size_t)batch * nb * DN_WIN;
   a.m32 = a.m8 + (size_t)batch * nb * DN_P;
-  a.mg = a.m32 + (size_t)batch * (nb / 4) * DN_P;
+  a.mc8 = reinterpret_cast<float2*>(a.m32 + (size_t)batch * (nb / 4) * DN_P);
+  a.mc32 = a.mc8 + (size_t)batch * nb * DN_BINS * DN_PC;
+  a.mg = reinterpret_cast<float*>(a.mc32 + (size_t)batch * (nb / 4) * DN_BINS * DN_PC);
   a.out = out;
   BART_CUDA(ctx, cudaFuncSetAttribute(dense_near_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(NearShared)));

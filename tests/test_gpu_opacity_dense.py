@@ -58,6 +58,25 @@ def test_dense_lists_match_the_oracle(ctx, N, dnu, cutoff, lines):
     assert e < MAX_REL and l2 < L2_REL
 
 
+@pytest.mark.parametrize("ratio", [1.0, 1.3, 3.9, 6.0])
+def test_wide_lorentz_profiles(ctx, ratio):
+    """Widths from a few grid points to a sixth of the cutoff and beyond, with
+    gamma_ref over one bin, several, and more than the kernels have bins for."""
+    import paper_2104_12522_gb300 as bart
+    N, dnu = 200, 0.02
+    species = [_list(0, 11_000, 970.0, 1034.0, dnu, 3)]
+    rng = np.random.default_rng(4)
+    g = 0.1 * ratio ** -rng.uniform(0.0, 1.0, species[0].n)
+    species[0] = W.LineList(species[0].nu0, species[0].log10_s296, species[0].elow, g.astype(np.float32), 18.0)
+    p, t = np.array([(1.2, 1500.0), (2.5, 3000.0), (5.0, 1500.0), (12.0, 900.0), (40.0, 1500.0), (100.0, 600.0)]).T
+    got = ctx.opacity_cells([bart.device_lines(s) for s in species], p, t, bart.NuGrid(1000.0, dnu, N), 25.0)
+    ctx.sync()
+    ref = O.opacity_cells(species, p, t, 1000.0, dnu, N, 25.0)
+    e, l2 = opacity_errors(got.cpu().numpy(), ref)
+    print(f"gamma_ref ratio {ratio}: max rel {e:.2e}, L2 {l2:.2e}")
+    assert e < MAX_REL and l2 < L2_REL
+
+
 def test_dense_and_line_by_line_agree(ctx):
     """The same list whole (dense) and in parts too thin for the dense path,
     added up in FP64; with and without the line-strength bound."""
