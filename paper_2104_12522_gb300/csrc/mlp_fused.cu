@@ -16,7 +16,7 @@
 //
 // Layout.  Features run along M (the 128 lanes of an accumulator), batch rows
 // along N: a CTA with few rows still fills the tensor core's M, the accumulator
-// of a layer is 4 R columns, and a thread owns one feature of all R rows, so
+// of a layer is 4 R columns, and a thread owns one feature of 8 rows (16 of 32), so
 // bias, GELU and the split into BF16 hi + lo stay in its registers.  A layer's
 // B operand holds the rows' hi parts and lo parts side by side (N = 2 R), so
 // one MMA multiplies the weights with both and the epilogue adds them.  The
@@ -28,8 +28,9 @@
 // (features by batch rows), which is what the weight gradients multiply.
 //
 // R is the smallest of 8, 16, 32 that gives every tile its own SM.
-// Measured (9-256-256-256-10): 2,048 rows 71.7 us layer by layer, 22.8 us
-// here; a training step on 1,024 rows 250 us and 70 us.
+// Measured (9-256-256-256-10): 2,048 rows 71.7 us layer by layer, 18.4 us here
+// (22.8 us with one thread to a feature of all rows and erff); a training step
+// on 1,024 rows 250 us and 67 us.
 #include <algorithm>
 #include <cmath>
 
@@ -37,8 +38,11 @@
 
 namespace {
 
-constexpr int MF_EPI = 256;                      // epilogue threads: one per feature
-constexpr int MF_THREADS = MF_EPI + 64;          // + producer warp + MMA warp
+// Epilogue threads: 256 per group of 8 rows (16 of 32), one per feature; then
+// the producer warp and the MMA warp.
+__host__ __device__ constexpr int mf_rows_per_thread(int R) { return R == 32 ? 16 : 8; }
+__host__ __device__ constexpr int mf_groups(int R) { return R / mf_rows_per_thread(R); }
+__host__ __device__ constexpr int mf_threads(int R) { return 256 * mf_groups(R) + 64; }
 constexpr int MF_STAGES = 4;
 constexpr unsigned int MF_BLOCK_BYTES = MF_WIDTH * 64 * 2;   // weights of one 64-deep K block
 constexpr unsigned int MF_SPIN_LIMIT = 1u << 22;             // try_wait rounds before a wait is given up
@@ -129,20 +133,31 @@ __device__ __forceinline__ void mma_commit(unsigned long long* b) {
 // N consecutive accumulator columns of this thread's TMEM lane.
 template <int N>
 __device__ __forceinline__ void tmem_load(unsigned int addr, float (&v)[N]) {
-  static_assert(N % 16 == 0, "");
-#pragma unroll
-  for (int c = 0; c < N; c += 16) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(addr + c)
-        : "memory");
+  static_assert(N == 8 || N % 16 == 0, "");
+  if constexpr (N == 8) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr)
+                 : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int q = 0; q < 16; ++q) v[c + q] = __uint_as_float(r[q]);
+    for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < N; c += 16) {
+      uint32_t r[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+          "%15}, [%16];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+            "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(addr + c)
+          : "memory");
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int q = 0; q < 16; ++q) v[c + q] = __uint_as_float(r[q]);
+    }
   }
 }
 
@@ -174,26 +189,60 @@ __device__ __forceinline__ unsigned int split_word(float v) {
   return (unsigned int)__bfloat16_as_ushort(h) | ((unsigned int)__bfloat16_as_ushort(l) << 16);
 }
 
+// The normal distribution function Phi(x) and, for the gradient, exp(-x^2 / 2):
+// Phi(-|x|) = erfc(z) / 2, z = |x| / sqrt 2, with erfc(z) = exp(-z^2) t P(t),
+// t = 1 / (1 + 0.3 z), P fitted by least squares (reweighted towards the largest
+// error) to 2.1e-8 relative over z <= 12.  Relative error of x Phi(x) in FP32
+// 1.4e-6 for |x| <= 5, absolute 3.8e-7 (erff: 4.5e-7, without the relative
+// accuracy below zero); no branch, a third of erff's instructions.
+__device__ __forceinline__ float normal_cdf(float x, float& e) {
+  const float ax = fabsf(x);
+  float t;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(ax, 0.3f * 0.70710678118654752f, 1.0f)));
+  float p = -0.12925601f;
+  p = fmaf(p, t, 0.484315053f);
+  p = fmaf(p, t, -0.50979936f);
+  p = fmaf(p, t, 0.544997127f);
+  p = fmaf(p, t, -0.0928463923f);
+  p = fmaf(p, t, 0.214189869f);
+  p = fmaf(p, t, 0.148519151f);
+  p = fmaf(p, t, 0.170691216f);
+  p = fmaf(p, t, 0.169189338f);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(ax * ax * -0.72134752044448170f));
+  const float tail = 0.5f * t * p * e;
+  return x >= 0.0f ? 1.0f - tail : tail;
+}
+__device__ __forceinline__ float mf_gelu(float x) {
+  float e;
+  return x * normal_cdf(x, e);
+}
+__device__ __forceinline__ float mf_gelu_grad(float x) {
+  float e;
+  const float c = normal_cdf(x, e);
+  return fmaf(x * 0.3989422804014327f, e, c);
+}
+
 template <int R, bool TRAIN>
-__global__ void __launch_bounds__(MF_THREADS, 1)
+__global__ void __launch_bounds__(mf_threads(R), 1)
 mlp_rows_kernel(const __grid_constant__ MfArgs a) {
   static_assert(R == 8 || R == 16 || R == 32, "");
   constexpr int N = 2 * R;                       // hi parts of the rows, then lo parts
+  constexpr int RT = mf_rows_per_thread(R), EPI = 256 * mf_groups(R);   // rows a thread, epilogue threads
   constexpr unsigned int B_SBO = 128, B_LBO = (N / 8) * 128;
   constexpr unsigned int TMEM_COLS = 2 * N;      // two halves of 128 features; a power of two >= 32
   constexpr unsigned int IDESC = um_idesc(128, N);
   extern __shared__ __align__(1024) unsigned char mf_smem[];
   unsigned char* ring = mf_smem;                                     // [MF_STAGES][MF_BLOCK_BYTES]
   unsigned char* opnd = mf_smem + MF_STAGES * MF_BLOCK_BYTES;        // B operand: K up to 256 x N, BF16
-  float* bacc = reinterpret_cast<float*>(opnd + (MF_WIDTH / 8) * B_LBO);   // [n_bias] (training)
+  float* bacc = reinterpret_cast<float*>(opnd + (MF_WIDTH / 8) * B_LBO);   // [row group][n_bias] (training)
   __shared__ __align__(8) unsigned long long full[MF_STAGES], empty[MF_STAGES], acc_bar, in_bar;
   __shared__ unsigned int s_tmem;
   __shared__ volatile int s_fail;
-  __shared__ double s_loss[MF_EPI / 32];
+  __shared__ double s_loss[EPI / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int L = a.n.L, steps = TRAIN ? 2 * L - 1 : L;
 
-  if (warp == MF_EPI / 32 + 1) {
+  if (warp == EPI / 32 + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_u32(&s_tmem)),
                  "r"(TMEM_COLS)
                  : "memory");
@@ -205,7 +254,7 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
       bar_init(&empty[q], 1);
     }
     bar_init(&acc_bar, 1);
-    bar_init(&in_bar, MF_EPI);
+    bar_init(&in_bar, EPI);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
@@ -214,7 +263,7 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned int tmem = s_tmem;
 
-  if (warp == MF_EPI / 32) {
+  if (warp == EPI / 32) {
     // ---- producer: the K blocks of every step of every tile, in order
     if (lane == 0) {
       unsigned int q = 0;
@@ -242,7 +291,7 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
           bar_wait(&full[i % MF_STAGES], (i / MF_STAGES) & 1u, &none);
       }
     }
-  } else if (warp == MF_EPI / 32 + 1) {
+  } else if (warp == EPI / 32 + 1) {
     // ---- MMA: one thread issues
     if (lane == 0) {
       unsigned int q = 0, done = 0;
@@ -278,23 +327,25 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
         }
     }
   } else {
-    // ---- epilogue: thread = feature, its R rows in registers
-    const int f = tid, half = warp >> 2;
-    const unsigned int t_addr = tmem + ((unsigned int)((warp & 3) * 32) << 16) + (unsigned int)(half * N);
+    // ---- epilogue: thread = feature, RT rows from r0 in registers (warp & 3 is
+    // the quadrant of TMEM lanes that a warp can read)
+    const int f = tid & 255, half = (warp >> 2) & 1, rg = tid >> 8, r0 = rg * RT;
+    const unsigned int t_addr = tmem + ((unsigned int)((warp & 3) * 32) << 16) + (unsigned int)(half * N + r0);
     const int g = (lane >> 3) & 3;
-    unsigned char* const my_opnd = opnd + (f >> 3) * B_LBO + (f & 7) * 2;
+    unsigned char* const my_opnd = opnd + (f >> 3) * B_LBO + (r0 / 8) * 128 + (f & 7) * 2;
+    float* const my_bacc = bacc + rg * a.n.n_bias;
     unsigned int done = 0;
     double loss = 0.0;
     const int n_in = a.n.w[0], n_out = a.n.w[L];
     if (TRAIN)
-      for (int l = 0; l < L; ++l)                // bias_at[l] + f belongs to thread f alone
-        if (f < a.n.w[l + 1]) bacc[a.n.bias_at[l] + f] = 0.0f;
+      for (int l = 0; l < L; ++l)                // bias_at[l] + f of a row group belongs to one thread
+        if (f < a.n.w[l + 1]) my_bacc[a.n.bias_at[l] + f] = 0.0f;
     // B operand of the next step, K = f: the rows' hi and lo parts.  The eight
     // rows of a core matrix are stored starting at a row that depends on the
     // lane's core matrix, so a warp's stores meet 32 different banks' words.
-    auto put = [&](const unsigned int (&w)[R]) {
+    auto put = [&](const unsigned int (&w)[RT]) {
 #pragma unroll
-      for (int q = 0; q < R / 8; ++q) {
+      for (int q = 0; q < RT / 8; ++q) {
         unsigned int u[8], v[8];
 #pragma unroll
         for (int s = 0; s < 8; ++s) u[s] = (g & 1) ? w[8 * q + ((s + 2) & 7)] : w[8 * q + s];
@@ -309,9 +360,9 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
       }
     };
     // the same values as an image for the weight gradients, K = batch rows
-    auto put_image = [&](long long at, int rows, long long b0, const unsigned int (&w)[R]) {
+    auto put_image = [&](long long at, int rows, long long b0, const unsigned int (&w)[RT]) {
 #pragma unroll
-      for (int q = 0; q < R / 8; ++q) {
+      for (int q = 0; q < RT / 8; ++q) {
         unsigned int h[4], l[4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
@@ -329,29 +380,30 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
       bar_arrive(&in_bar);
     };
     // waits for the step's accumulator; v = its hi and lo products added
-    auto take = [&](int m, float (&v)[R]) -> bool {
+    auto take = [&](int m, float (&v)[RT]) -> bool {
       if (!__all_sync(0xffffffffu, bar_wait(&acc_bar, done & 1u, &s_fail))) return false;
       ++done;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (half * 128 < m) {                      // uniform over the warp
-        float d[N];
-        tmem_load<N>(t_addr, d);
+        float d[RT];
+        tmem_load<RT>(t_addr, v);
+        tmem_load<RT>(t_addr + R, d);
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = d[r] + d[R + r];
+        for (int r = 0; r < RT; ++r) v[r] += d[r];
       } else {
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = 0.0f;
+        for (int r = 0; r < RT; ++r) v[r] = 0.0f;
       }
       return true;
     };
 
     bool ok = true;
     for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x) {
-      const int64_t b0 = (int64_t)tile * R;
-      unsigned int w[R];
+      const int64_t b0 = (int64_t)tile * R + r0;   // the thread's first row
+      unsigned int w[RT];
       if (f < pad_to(n_in, 16)) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
+        for (int r = 0; r < RT; ++r) {
           float v = 0.0f;
           if (f < n_in && b0 + r < a.B) {
             int64_t row = b0 + r;
@@ -370,22 +422,38 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
         if (TRAIN) put_image(a.n.ht[0], pad_to(n_in, 16), b0, w);
       }
       publish();
-      float v[R];
+      float v[RT];
       for (int l = 0; ok && l < L; ++l) {
         const int m = a.n.w[l + 1];
+        // what the epilogue reads from memory is requested before the wait
+        const float bias = f < m ? a.p[a.n.b_off[l] + f] : 0.0f;
+        float target[RT];
+        if (TRAIN && l + 1 == L) {
+#pragma unroll
+          for (int r = 0; r < RT; ++r) {
+            target[r] = 1.0f;
+            if (f < m && b0 + r < a.B) {
+              int64_t row = b0 + r;
+              if (a.rows) {
+                row = a.rows[b0 + r];
+                if (row < 0 || row >= a.n_rows) row = 0;
+              }
+              target[r] = a.t[row * m + f];
+            }
+          }
+        }
         if (!take(m, v)) {
           ok = false;
           break;
         }
-        const float bias = f < m ? a.p[a.n.b_off[l] + f] : 0.0f;
         if (l + 1 < L) {
           if (f < pad_to(m, 16)) {
             float* z = TRAIN ? a.z + a.n.z[l + 1] + b0 * m + f : nullptr;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
+            for (int r = 0; r < RT; ++r) {
               const float zz = v[r] + bias;
               if (TRAIN && f < m) z[(int64_t)r * m] = zz;
-              w[r] = f < m ? split_word(gelu(zz)) : 0u;
+              w[r] = f < m ? split_word(mf_gelu(zz)) : 0u;
             }
             put(w);
             if (TRAIN) put_image(a.n.ht[l + 1], pad_to(m, 16), b0, w);
@@ -395,7 +463,7 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
           if (f < m) {
             const float osh = a.scale[2 * n_in + f], osc = a.scale[2 * n_in + n_out + f];
 #pragma unroll
-            for (int r = 0; r < R; ++r)
+            for (int r = 0; r < RT; ++r)
               if (b0 + r < a.B) {
                 const float s = (v[r] + bias) / osc + osh;
                 a.y[(b0 + r) * m + f] = a.log_outputs ? exp10f(s) : s;
@@ -405,15 +473,10 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
           // the gradient of the loss by the standardised output
           float db = 0.0f;
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
+          for (int r = 0; r < RT; ++r) {
             float dy = 0.0f;
             if (f < m && b0 + r < a.B) {
-              int64_t row = b0 + r;
-              if (a.rows) {
-                row = a.rows[b0 + r];
-                if (row < 0 || row >= a.n_rows) row = 0;
-              }
-              const float tv = a.t[row * m + f], ts = a.log_outputs ? log10f(tv) : tv;
+              const float tv = target[r], ts = a.log_outputs ? log10f(tv) : tv;
               const float e = (v[r] + bias) - (ts - a.scale[2 * n_in + f]) * a.scale[2 * n_in + n_out + f];
               dy = a.inv * e;
               loss += (double)e * e;
@@ -423,39 +486,38 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
           }
           put(w);
           put_image(a.n.dt[l], pad_to(m, 128), b0, w);
-          if (f < m) bacc[a.n.bias_at[l] + f] += db;
+          if (f < m) my_bacc[a.n.bias_at[l] + f] += db;
         }
       }
       if (TRAIN && ok && L > 1) {
         publish();
         for (int l = L - 1; l >= 1; --l) {       // dz of layer l-1 from dz of layer l
           const int m = a.n.w[l];
+          float z[RT];
+#pragma unroll
+          for (int r = 0; r < RT; ++r) z[r] = f < m ? a.z[a.n.z[l] + (b0 + r) * m + f] : 0.0f;   // this thread's own, from above
           if (!take(m, v)) {
             ok = false;
             break;
           }
           if (f < pad_to(m, 16)) {
-            const float* z = a.z + a.n.z[l] + b0 * m + f;   // written by this thread above
             float db = 0.0f;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
+            for (int r = 0; r < RT; ++r) {
               // rows past the batch carry zeros
-              const float dz = f < m ? v[r] * gelu_grad(z[(int64_t)r * m]) : 0.0f;
+              const float dz = f < m ? v[r] * mf_gelu_grad(z[r]) : 0.0f;
               db += dz;
               w[r] = split_word(dz);
             }
             if (l > 1) put(w);
             put_image(a.n.dt[l - 1], pad_to(m, 128), b0, w);
-            if (f < m) bacc[a.n.bias_at[l - 1] + f] += db;
+            if (f < m) my_bacc[a.n.bias_at[l - 1] + f] += db;
           }
           if (l > 1) publish();
         }
       }
     }
     if (TRAIN && ok) {
-      for (int l = 0; l < L; ++l)
-        if (f < a.n.w[l + 1])
-          a.bpart[(int64_t)blockIdx.x * a.n.n_bias + a.n.bias_at[l] + f] = bacc[a.n.bias_at[l] + f];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
       if (lane == 0) s_loss[warp] = loss;
@@ -470,11 +532,17 @@ mlp_rows_kernel(const __grid_constant__ MfArgs a) {
       atomicOr(a.status, BART_DEV_TIMEOUT);
     } else if (TRAIN) {
       double s = 0.0;
-      for (int q = 0; q < MF_EPI / 32; ++q) s += s_loss[q];
+      for (int q = 0; q < EPI / 32; ++q) s += s_loss[q];
       a.lpart[blockIdx.x] = s;
     }
   }
-  if (warp == MF_EPI / 32 + 1)
+  if (TRAIN && !s_fail)
+    for (int q = tid; q < a.n.n_bias; q += blockDim.x) {
+      float s = bacc[q];
+      for (int g = 1; g < mf_groups(R); ++g) s += bacc[g * a.n.n_bias + q];
+      a.bpart[(int64_t)blockIdx.x * a.n.n_bias + q] = s;
+    }
+  if (warp == EPI / 32 + 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
@@ -707,13 +775,13 @@ int max_ctas(const bart_mlp* net) { return net->ctx->sm_count; }   // one reside
 template <int R, bool TRAIN>
 cudaError_t launch_rows(bart_mlp* net, MfArgs& a, int64_t rows, int* ctas) {
   const size_t smem = (size_t)MF_STAGES * MF_BLOCK_BYTES + (size_t)(MF_WIDTH / 8) * (2 * R / 8) * 128 +
-                      (TRAIN ? (size_t)a.n.n_bias * sizeof(float) : 0);
+                      (TRAIN ? (size_t)mf_groups(R) * a.n.n_bias * sizeof(float) : 0);
   cudaError_t e = cudaFuncSetAttribute(mlp_rows_kernel<R, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
   a.tiles = (int)((rows + R - 1) / R);
   *ctas = std::min(a.tiles, max_ctas(net));
-  mlp_rows_kernel<R, TRAIN><<<*ctas, MF_THREADS, smem, net->ctx->stream>>>(a);
+  mlp_rows_kernel<R, TRAIN><<<*ctas, mf_threads(R), smem, net->ctx->stream>>>(a);
   return cudaGetLastError();
 }
 
