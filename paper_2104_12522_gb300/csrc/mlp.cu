@@ -347,7 +347,9 @@ umma_gemm_kernel(int M, int N, int K, int k_per, const TA* __restrict__ A, int64
           }
         } else {
           const int64_t o = (int64_t)gm * ldc + nb;
-          const bool vec = nb + 32 <= N && (ldc & 3) == 0;
+          // (the rows of an odd batch or of a layer behind odd widths may start anywhere)
+          const uintptr_t at = reinterpret_cast<uintptr_t>(C + o) | (mode == 1 ? reinterpret_cast<uintptr_t>(H + o) : 0);
+          const bool vec = nb + 32 <= N && (at & 15) == 0;
           if (mode == 1 || mode == 2) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) x[j] += (nb + j < N) ? bias[nb + j] : 0.0f;
