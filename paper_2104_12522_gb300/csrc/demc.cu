@@ -34,7 +34,7 @@
 #include <cmath>
 #include <vector>
 
-#include "bart_internal.cuh"
+#include "demc.cuh"
 
 struct bart_demc {
   bart_ctx* ctx = nullptr;
@@ -91,11 +91,19 @@ __device__ __forceinline__ void half_range(int C, int h, int& b, int& e) {
   e = h ? C : c0;
 }
 
-__global__ void propose_kernel(int C, int d, const float* __restrict__ x, const float* __restrict__ lo,
-                               const float* __restrict__ hi, int64_t gen_arg, const int64_t* __restrict__ gen_dev,
-                               uint64_t seed, double gamma, int jump_every, double eps, float* __restrict__ y,
-                               int32_t* __restrict__ inbox) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per chain, a lane per parameter (at most 32): the FP64 logarithm, root
+// and cosine of a parameter's noise are a long serial chain, and one thread per
+// chain walked the parameters one after the other (16 chains x 9 parameters:
+// 29 us, 5 us with the lanes).  Every value is formed as before.
+constexpr int WARPS = 4;                      // chains per CTA of the warp-per-chain kernels
+__device__ __forceinline__ int warp_chain() { return blockIdx.x * WARPS + (threadIdx.x >> 5); }
+
+__global__ void __launch_bounds__(32 * WARPS)
+propose_kernel(int C, int d, const float* __restrict__ x, const float* __restrict__ lo,
+               const float* __restrict__ hi, int64_t gen_arg, const int64_t* __restrict__ gen_dev,
+               uint64_t seed, double gamma, int jump_every, double eps, float* __restrict__ y,
+               int32_t* __restrict__ inbox) {
+  const int i = warp_chain(), q = threadIdx.x & 31;
   if (i >= C) return;
   const int64_t gen = gen_dev ? *gen_dev : gen_arg;
   const int h = (int)(gen & 1);               // half updated this half-step
@@ -103,8 +111,8 @@ __global__ void propose_kernel(int C, int d, const float* __restrict__ x, const 
   half_range(C, h, b, e);
   half_range(C, 1 - h, ob, oe);
   if (i < b || i >= e) {                      // not updated: copy, mark inactive
-    for (int q = 0; q < d; ++q) y[(int64_t)i * d + q] = x[(int64_t)i * d + q];
-    inbox[i] = 0;
+    if (q < d) y[(int64_t)i * d + q] = x[(int64_t)i * d + q];
+    if (q == 0) inbox[i] = 0;
     return;
   }
   const int no = oe - ob;
@@ -113,26 +121,29 @@ __global__ void propose_kernel(int C, int d, const float* __restrict__ x, const 
   if (r2 >= r1) ++r2;
   const int64_t g2 = gen >> 1;                // generation index (two half-steps each)
   const double gm = (jump_every > 0 && (g2 % jump_every) == jump_every - 1) ? 1.0 : gamma;
-  int ok = 1;
-  for (int q = 0; q < d; ++q) {
+  bool ok = true;
+  if (q < d) {
     const double w = (double)hi[q] - (double)lo[q];
     const double v = (double)x[(int64_t)i * d + q] +
                      gm * ((double)x[(int64_t)r1 * d + q] - (double)x[(int64_t)r2 * d + q]) +
                      eps * w * normal(seed, gen, i, 8 + q);
     const float vf = (float)v;
     y[(int64_t)i * d + q] = vf;
-    ok &= (vf >= lo[q]) && (vf <= hi[q]);
+    ok = (vf >= lo[q]) && (vf <= hi[q]);
   }
-  inbox[i] = ok;
+  ok = __all_sync(0xffffffffu, ok);
+  if (q == 0) inbox[i] = ok;
 }
 
-// DEMCzs proposals: all chains, from the archive.
-__global__ void propose_zs_kernel(int C, int d, const float* __restrict__ x, const float* __restrict__ lo,
-                                  const float* __restrict__ hi, int64_t gen_arg, const int64_t* __restrict__ gen_dev,
-                                  uint64_t seed, double gamma, int jump_every, double eps, const float* __restrict__ Z,
-                                  const long long* __restrict__ zc, double p_snooker, float* __restrict__ y,
-                                  int32_t* __restrict__ inbox, double* __restrict__ logq) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// DEMCzs proposals: all chains, from the archive.  The snooker move's sums run
+// over the parameters in order in every lane.
+__global__ void __launch_bounds__(32 * WARPS)
+propose_zs_kernel(int C, int d, const float* __restrict__ x, const float* __restrict__ lo,
+                  const float* __restrict__ hi, int64_t gen_arg, const int64_t* __restrict__ gen_dev,
+                  uint64_t seed, double gamma, int jump_every, double eps, const float* __restrict__ Z,
+                  const long long* __restrict__ zc, double p_snooker, float* __restrict__ y,
+                  int32_t* __restrict__ inbox, double* __restrict__ logq) {
+  const int i = warp_chain(), lane = threadIdx.x & 31;
   if (i >= C) return;
   const int64_t gen = gen_dev ? *gen_dev : gen_arg;
   const int m = (int)*zc;
@@ -143,7 +154,7 @@ __global__ void propose_zs_kernel(int C, int d, const float* __restrict__ x, con
   const float* za = Z + (int64_t)a * d;
   const float* zb = Z + (int64_t)b * d;
   double lq = 0.0;
-  int ok = 1;
+  bool ok = true;
   if (uniform(seed, gen, i, 50) < p_snooker) {
     const int c = min((int)(uniform(seed, gen, i, 53) * m), m - 1);
     const float* zz = Z + (int64_t)c * d;
@@ -154,8 +165,8 @@ __global__ void propose_zs_kernel(int C, int d, const float* __restrict__ x, con
       proj += ((double)za[q] - zb[q]) * e;
     }
     if (nn == 0.0) {                          // x on an archive state: no move
-      ok = 0;
-      for (int q = 0; q < d; ++q) y[(int64_t)i * d + q] = xi[q];
+      ok = false;
+      if (lane < d) y[(int64_t)i * d + lane] = xi[lane];
     } else {
       const double gs = 1.2 + uniform(seed, gen, i, 54);
       const double f = gs * proj / nn;
@@ -163,8 +174,8 @@ __global__ void propose_zs_kernel(int C, int d, const float* __restrict__ x, con
       for (int q = 0; q < d; ++q) {
         const double e = (double)xi[q] - zz[q];
         const float vf = (float)((double)xi[q] + f * e);
-        y[(int64_t)i * d + q] = vf;
-        ok &= (vf >= lo[q]) && (vf <= hi[q]);
+        if (lane == q) y[(int64_t)i * d + q] = vf;
+        ok = ok && (vf >= lo[q]) && (vf <= hi[q]);
         const double dy = (double)vf - zz[q];
         ny += dy * dy;
       }
@@ -172,15 +183,19 @@ __global__ void propose_zs_kernel(int C, int d, const float* __restrict__ x, con
     }
   } else {
     const double gm = (jump_every > 0 && (gen % jump_every) == jump_every - 1) ? 1.0 : gamma;
-    for (int q = 0; q < d; ++q) {
+    if (lane < d) {
+      const int q = lane;
       const double w = (double)hi[q] - (double)lo[q];
       const float vf = (float)((double)xi[q] + gm * ((double)za[q] - zb[q]) + eps * w * normal(seed, gen, i, 8 + q));
       y[(int64_t)i * d + q] = vf;
-      ok &= (vf >= lo[q]) && (vf <= hi[q]);
+      ok = (vf >= lo[q]) && (vf <= hi[q]);
     }
+    ok = __all_sync(0xffffffffu, ok);
   }
-  inbox[i] = ok;
-  logq[i] = lq;
+  if (lane == 0) {
+    inbox[i] = ok;
+    logq[i] = lq;
+  }
 }
 
 // Appends the chains' states to the archive every `thin` steps while it has room.
@@ -246,25 +261,137 @@ __global__ void accept_kernel(int C, int d, float* __restrict__ x, double* __res
   if (accepted) accepted[i] = a;
 }
 
-// out[i] = -1/2 sum_b ((m_ib - d_b) / s_b)^2 in FP64; -inf where mask[i] == 0.
-__global__ void loglike_kernel(const float* __restrict__ m, int n, int nb, const float* __restrict__ data,
-                               const float* __restrict__ sigma, const int32_t* __restrict__ mask,
-                               double* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (mask && !mask[i]) {
-    out[i] = -INFINITY;
-    return;
-  }
+// -1/2 sum_b ((m_b - d_b) / s_b)^2 in FP64 of one model's band values, by a warp:
+// the lanes take the bands' divisions, the sum runs over the bands in order in
+// every lane.
+__device__ double warp_loglike(const float* __restrict__ m, int nb, const float* __restrict__ data,
+                               const float* __restrict__ sigma) {
+  const int lane = threadIdx.x & 31;
   double s = 0.0;
-  for (int b = 0; b < nb; ++b) {
-    const double r = ((double)m[(int64_t)i * nb + b] - (double)data[b]) / (double)sigma[b];
-    s += r * r;
+  for (int b0 = 0; b0 < nb; b0 += 32) {
+    double r = 0.0;
+    if (b0 + lane < nb) r = ((double)m[b0 + lane] - (double)data[b0 + lane]) / (double)sigma[b0 + lane];
+    for (int b = 0; b < min(32, nb - b0); ++b) {
+      const double rb = __shfl_sync(0xffffffffu, r, b);
+      s += rb * rb;
+    }
   }
-  out[i] = -0.5 * s;
+  return -0.5 * s;
+}
+
+// out[i] = the log-likelihood of row i; -inf where mask[i] == 0.
+__global__ void __launch_bounds__(32 * WARPS)
+loglike_kernel(const float* __restrict__ m, int n, int nb, const float* __restrict__ data,
+               const float* __restrict__ sigma, const int32_t* __restrict__ mask, double* __restrict__ out) {
+  const int i = warp_chain();
+  if (i >= n) return;
+  double v = -INFINITY;
+  if (!mask || mask[i]) v = warp_loglike(m + (int64_t)i * nb, nb, data, sigma);
+  if ((threadIdx.x & 31) == 0) out[i] = v;
+}
+
+// A half-step of the retrieval loop in two launches around the forward model
+// (they were seven: log-likelihoods, screen, acceptance, archive, statistics
+// and the counter, 2 to 8 us each).
+// Before it: the surrogate's log-likelihoods and the screen.
+__global__ void __launch_bounds__(32 * WARPS)
+screen_bands_kernel(int C, int nb, const int32_t* __restrict__ inbox, const float* __restrict__ bs,
+                    const float* __restrict__ data, const float* __restrict__ sigma, double* __restrict__ lsy,
+                    const double* __restrict__ ls_x, const int64_t* __restrict__ gen_dev, uint64_t seed, double beta,
+                    double margin, const double* __restrict__ logq, int32_t* __restrict__ pass) {
+  const int i = warp_chain();
+  if (i >= C) return;
+  int p = inbox[i];
+  if (bs) {
+    double v = -INFINITY;
+    if (p) {
+      v = warp_loglike(bs + (int64_t)i * nb, nb, data, sigma);
+      const double lu = log(uniform(seed, *gen_dev, i, 100));
+      p = lu < log_a1(v - ls_x[i], beta, margin, logq ? logq[i] : 0.0);
+    }
+    if ((threadIdx.x & 31) == 0) lsy[i] = v;
+  }
+  if ((threadIdx.x & 31) == 0) pass[i] = p;
+}
+
+// After it: the exact log-likelihoods, the acceptance and state update, and the
+// statistics; the last CTA to finish appends to the DEMCzs archive and advances
+// the half-step counter.
+__global__ void __launch_bounds__(32 * WARPS)
+finish_kernel(int C, int d, int nb, float* __restrict__ x, double* __restrict__ L, double* __restrict__ Ls,
+              const float* __restrict__ y, const int32_t* __restrict__ inbox, const int32_t* __restrict__ pass,
+              const float* __restrict__ be, const float* __restrict__ bs, const double* __restrict__ lsy,
+              const float* __restrict__ data, const float* __restrict__ sigma, int64_t* hs, uint64_t seed,
+              double beta, double margin, const double* __restrict__ logq, int thin, float* __restrict__ Z,
+              int64_t cap, long long* __restrict__ zc, DemcStats* __restrict__ st, unsigned int* __restrict__ done) {
+  __shared__ int s_last;
+  const int i = warp_chain(), lane = threadIdx.x & 31;
+  const int64_t gen = *hs;
+  if (i < C) {
+    const int in = inbox[i], p = pass[i];
+    bool a = false;
+    double Ly = 0.0;
+    if (p) {
+      Ly = warp_loglike(be + (int64_t)i * nb, nb, data, sigma);
+      const double lq = logq ? logq[i] : 0.0;
+      double r = Ly - L[i] + lq;
+      if (bs) {
+        const double dl = lsy[i] - Ls[i];       // as accept_kernel
+        r += log_a1(-dl, beta, margin, -lq) - log_a1(dl, beta, margin, lq);
+      }
+      const double lu = log(uniform(seed, gen, i, 101));
+      a = ((r >= 0.0) || (lu < r)) && Ly == Ly; // a NaN likelihood is never accepted
+    }
+    __syncwarp();                               // every lane has read L and Ls
+    if (a) {
+      if (lane < d) x[(int64_t)i * d + lane] = y[(int64_t)i * d + lane];
+      if (lane == 0) {
+        L[i] = Ly;
+        if (bs) Ls[i] = lsy[i];
+      }
+      if (bs) {                                 // the surrogate's band error on accepted samples
+        float e = 0.f;
+        for (int b = lane; b < nb; b += 32) {
+          const float ref = be[(int64_t)i * nb + b];
+          e = fmaxf(e, fabsf(bs[(int64_t)i * nb + b] - ref) / fabsf(ref));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+        if (lane == 0) {
+          atomicAdd(&st->err_sum, (double)e);
+          atomicMax(&st->err_max_bits, __float_as_uint(e));
+        }
+      }
+    }
+    if (lane == 0) {
+      if (in) atomicAdd(&st->proposals, 1ULL);
+      if (in && !p) atomicAdd(&st->screened_out, 1ULL);
+      if (p) atomicAdd(&st->exact_evals, 1ULL);
+      if (a) atomicAdd(&st->accepted, 1ULL);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) + 1u == gridDim.x;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();                              // the other CTAs' states are visible
+  if (Z) {
+    const long long m = *zc;
+    if ((gen + 1) % thin == 0 && m + C <= cap) {
+      for (int64_t e = threadIdx.x; e < (int64_t)C * d; e += blockDim.x) Z[m * d + e] = __ldcg(x + e);
+      __syncthreads();
+      if (threadIdx.x == 0) *zc = m + C;
+    }
+  }
+  if (threadIdx.x == 0) {
+    *done = 0u;
+    *hs = gen + 1;
+  }
 }
 
 unsigned nblk(int n) { return (unsigned)((n + 127) / 128); }
+unsigned nwarps(int n) { return (unsigned)((n + WARPS - 1) / WARPS); }   // CTAs of the warp-per-chain kernels
 
 }  // namespace
 
@@ -343,13 +470,13 @@ extern "C" bart_status bart_demc_propose(bart_demc* s, int64_t half_step, float*
   BART_REQUIRE(s->ctx, y && inbox, "NULL y or inbox");
   BART_REQUIRE(s->ctx, half_step >= 0, "half_step must be >= 0");
   if (s->zs) {
-    propose_zs_kernel<<<nblk(s->C), 128, 0, s->ctx->stream>>>(s->C, s->d, s->x, s->lo, s->hi, half_step, s->hs_dev,
+    propose_zs_kernel<<<nwarps(s->C), 32 * WARPS, 0, s->ctx->stream>>>(s->C, s->d, s->x, s->lo, s->hi, half_step, s->hs_dev,
                                                               s->seed, s->gamma, s->jump_every, s->eps, s->Z, s->zc,
                                                               s->p_snooker, y, inbox, s->logq);
     return bart_check_launch(s->ctx, "propose_zs_kernel");
   }
   BART_REQUIRE(s->ctx, s->C >= 6, "DE-MC needs at least 6 chains (3 per half); DEMCzs needs 3");
-  propose_kernel<<<nblk(s->C), 128, 0, s->ctx->stream>>>(s->C, s->d, s->x, s->lo, s->hi, half_step, s->hs_dev,
+  propose_kernel<<<nwarps(s->C), 32 * WARPS, 0, s->ctx->stream>>>(s->C, s->d, s->x, s->lo, s->hi, half_step, s->hs_dev,
                                                          s->seed, s->gamma, s->jump_every, s->eps, y, inbox);
   return bart_check_launch(s->ctx, "propose_kernel");
 }
@@ -382,7 +509,7 @@ extern "C" bart_status bart_loglike_bands(bart_ctx* ctx, const float* model, int
   if (!ctx) return BART_EINVAL;
   BART_REQUIRE(ctx, model && data && sigma && out, "NULL array");
   BART_REQUIRE(ctx, n >= 1 && n_bands >= 1, "n and n_bands must be >= 1");
-  loglike_kernel<<<nblk(n), 128, 0, ctx->stream>>>(model, n, n_bands, data, sigma, mask, out);
+  loglike_kernel<<<nwarps(n), 32 * WARPS, 0, ctx->stream>>>(model, n, n_bands, data, sigma, mask, out);
   return bart_check_launch(ctx, "loglike_kernel");
 }
 
@@ -399,6 +526,21 @@ void bart_demc_use_counter(bart_demc* s, const int64_t* hs_dev) { s->hs_dev = hs
 int bart_demc_chains(const bart_demc* s) { return s->C; }
 int bart_demc_params(const bart_demc* s) { return s->d; }
 const float* bart_demc_states(const bart_demc* s) { return s->x; }
+
+bart_status bart_demc_screen_bands(bart_demc* s, const DemcHalfStep& h) {
+  screen_bands_kernel<<<nwarps(s->C), 32 * WARPS, 0, s->ctx->stream>>>(
+      s->C, h.n_bands, h.inbox, h.bands_s, h.data, h.sigma, h.ls_y, s->Ls, s->hs_dev, s->seed, s->beta, s->margin,
+      s->zs ? s->logq : nullptr, h.pass);
+  return bart_check_launch(s->ctx, "screen_bands_kernel");
+}
+
+bart_status bart_demc_finish(bart_demc* s, const DemcHalfStep& h, int64_t* hs) {
+  finish_kernel<<<nwarps(s->C), 32 * WARPS, 0, s->ctx->stream>>>(
+      s->C, s->d, h.n_bands, s->x, s->L, s->Ls, h.y, h.inbox, h.pass, h.bands, h.bands_s, h.ls_y, h.data, h.sigma, hs,
+      s->seed, s->beta, s->margin, s->zs ? s->logq : nullptr, s->thin, s->zs ? s->Z : nullptr, s->cap, s->zc, h.stats,
+      h.done);
+  return bart_check_launch(s->ctx, "finish_kernel");
+}
 
 extern "C" bart_status bart_demc_set_archive(bart_demc* s, const float* z0, int64_t n0, int64_t capacity, int thin,
                                              double p_snooker) {

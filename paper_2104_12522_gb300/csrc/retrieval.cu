@@ -4,55 +4,20 @@
 // run natively, one generation per CUDA-graph launch.
 //
 // A generation is two half-steps.  Each half-step is, on the context's stream:
-//   propose -> [surrogate forward -> surrogate log-likelihood] -> screen ->
+//   propose -> [surrogate forward] -> surrogate log-likelihood and screen ->
 //   exact forward model of the survivors only (inactive proposals' CTAs exit
-//   at once) -> exact log-likelihood -> accept -> statistics,
-// followed by an increment of the device half-step counter that the sampler
-// kernels read, so the captured graph replays every generation unchanged.
+//   at once) -> exact log-likelihood, accept, statistics and an increment of
+//   the device half-step counter that the sampler kernels read,
+// five launches, so the captured graph replays every generation unchanged.
 // The first generation runs eagerly: it sizes the scratch buffers and uploads
 // the constant tables, after which the captured calls launch kernels only.
 #include <cmath>
 #include <cstring>
 #include <vector>
 
-#include "bart_internal.cuh"
-
-void bart_demc_use_counter(bart_demc* s, const int64_t* hs_dev);
-int bart_demc_chains(const bart_demc* s);
-int bart_demc_params(const bart_demc* s);
-const float* bart_demc_states(const bart_demc* s);
+#include "demc.cuh"
 
 namespace {
-
-struct DevStats {
-  unsigned long long proposals, screened_out, exact_evals, accepted;
-  double err_sum;
-  unsigned int err_max_bits;    // non-negative float, ordered as its bit pattern
-};
-
-__global__ void stats_kernel(int C, int nb, const int32_t* __restrict__ inbox, const int32_t* __restrict__ pass,
-                             const int32_t* __restrict__ acc, const float* __restrict__ bs,
-                             const float* __restrict__ be, DevStats* __restrict__ st) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= C) return;
-  if (inbox[i]) atomicAdd(&st->proposals, 1ULL);
-  if (inbox[i] && !pass[i]) atomicAdd(&st->screened_out, 1ULL);
-  if (pass[i]) atomicAdd(&st->exact_evals, 1ULL);
-  if (acc[i]) {
-    atomicAdd(&st->accepted, 1ULL);
-    if (bs) {
-      float e = 0.f;
-      for (int b = 0; b < nb; ++b) {
-        const float ref = be[(int64_t)i * nb + b];
-        e = fmaxf(e, fabsf(bs[(int64_t)i * nb + b] - ref) / fabsf(ref));
-      }
-      atomicAdd(&st->err_sum, (double)e);
-      atomicMax(&st->err_max_bits, __float_as_uint(e));
-    }
-  }
-}
-
-__global__ void advance_kernel(int64_t* hs) { *hs += 1; }
 
 __global__ void record_kernel(const float* __restrict__ x, int n, const int64_t* __restrict__ hs, int64_t first,
                               float* __restrict__ chain) {
@@ -80,28 +45,27 @@ extern "C" bart_status bart_retrieval_run(bart_ctx* ctx, bart_demc* s, bart_mlp*
   BART_CUDA(ctx, cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
   bart_status r;
-  void *p_y, *p_inbox, *p_pass, *p_acc, *p_ly, *p_lsy, *p_be, *p_bs, *p_hs, *p_stats;
+  void *p_y, *p_inbox, *p_pass, *p_lsy, *p_be, *p_bs, *p_hs, *p_stats, *p_done;
   if ((r = bart_scratch(ctx, "rt_y", (size_t)C * d * 4, &p_y)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_inbox", (size_t)C * 4, &p_inbox)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_pass", (size_t)C * 4, &p_pass)) != BART_OK) return r;
-  if ((r = bart_scratch(ctx, "rt_acc", (size_t)C * 4, &p_acc)) != BART_OK) return r;
-  if ((r = bart_scratch(ctx, "rt_ly", (size_t)C * 8, &p_ly)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_lsy", (size_t)C * 8, &p_lsy)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_be", (size_t)C * nb * 4, &p_be)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_bs", (size_t)C * nb * 4, &p_bs)) != BART_OK) return r;
   if ((r = bart_scratch(ctx, "rt_hs", sizeof(int64_t), &p_hs)) != BART_OK) return r;
-  if ((r = bart_scratch(ctx, "rt_stats", sizeof(DevStats), &p_stats)) != BART_OK) return r;
+  if ((r = bart_scratch(ctx, "rt_stats", sizeof(DemcStats), &p_stats)) != BART_OK) return r;
+  if ((r = bart_scratch(ctx, "rt_done", sizeof(unsigned int), &p_done)) != BART_OK) return r;
   int64_t* hs = (int64_t*)p_hs;
-  float* y = (float*)p_y;
-  int32_t *inbox = (int32_t*)p_inbox, *pass = (int32_t*)p_pass, *acc = (int32_t*)p_acc;
-  double *ly = (double*)p_ly, *lsy = (double*)p_lsy;
-  float *be = (float*)p_be, *bs = (float*)p_bs;
+  float *y = (float*)p_y, *be = (float*)p_be, *bs = (float*)p_bs;
+  int32_t *inbox = (int32_t*)p_inbox, *pass = (int32_t*)p_pass;
+  const DemcHalfStep half{y, inbox, pass, nb, surrogate ? bs : nullptr, be, (double*)p_lsy, data, sigma,
+                          (DemcStats*)p_stats, (unsigned int*)p_done};
   // host staging copies live in the context's constant cache so the async
   // uploads read memory that outlives this call
   void* dummy;
   if ((r = bart_upload_const(ctx, "rt_hs_init", &first_half_step, sizeof(int64_t), &dummy)) != BART_OK) return r;
   BART_CUDA(ctx, cudaMemcpyAsync(hs, dummy, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
-  BART_CUDA(ctx, cudaMemsetAsync(p_stats, 0, sizeof(DevStats), st));
+  BART_CUDA(ctx, cudaMemsetAsync(p_stats, 0, sizeof(DemcStats), st));
   bart_demc_use_counter(s, hs);
 
   bart_batch batch{};
@@ -112,19 +76,10 @@ extern "C" bart_status bart_retrieval_run(bart_ctx* ctx, bart_demc* s, bart_mlp*
   auto half_step = [&]() -> bart_status {
     bart_status q;
     if ((q = bart_demc_propose(s, 0, y, inbox)) != BART_OK) return q;
-    if (surrogate) {
-      if ((q = bart_mlp_forward(surrogate, y, C, bs)) != BART_OK) return q;
-      if ((q = bart_loglike_bands(ctx, bs, C, nb, data, sigma, inbox, lsy)) != BART_OK) return q;
-    }
-    if ((q = bart_demc_screen(s, 0, inbox, surrogate ? lsy : nullptr, pass)) != BART_OK) return q;
+    if (surrogate && (q = bart_mlp_forward(surrogate, y, C, bs)) != BART_OK) return q;
+    if ((q = bart_demc_screen_bands(s, half)) != BART_OK) return q;
     if ((q = bart_forward_spectra_batch(ctx, grid, cfg, &batch, nullptr, filters, be)) != BART_OK) return q;
-    if ((q = bart_loglike_bands(ctx, be, C, nb, data, sigma, pass, ly)) != BART_OK) return q;
-    if ((q = bart_demc_accept(s, 0, y, pass, ly, surrogate ? lsy : nullptr, acc)) != BART_OK) return q;
-    // ctx->stream, not st: during capture it is the capture stream
-    stats_kernel<<<(C + 127) / 128, 128, 0, ctx->stream>>>(C, nb, inbox, pass, acc, surrogate ? bs : nullptr, be,
-                                                           (DevStats*)p_stats);
-    advance_kernel<<<1, 1, 0, ctx->stream>>>(hs);
-    return bart_check_launch(ctx, "retrieval half-step");
+    return bart_demc_finish(s, half, hs);
   };
   auto generation = [&]() -> bart_status {
     bart_status q;
@@ -191,8 +146,8 @@ extern "C" bart_status bart_retrieval_run(bart_ctx* ctx, bart_demc* s, bart_mlp*
   bart_demc_use_counter(s, nullptr);
   if (r != BART_OK) return r;
   if (stats) {
-    DevStats h{};
-    BART_CUDA(ctx, cudaMemcpyAsync(&h, p_stats, sizeof(DevStats), cudaMemcpyDeviceToHost, st));
+    DemcStats h{};
+    BART_CUDA(ctx, cudaMemcpyAsync(&h, p_stats, sizeof(DemcStats), cudaMemcpyDeviceToHost, st));
     BART_CUDA(ctx, cudaStreamSynchronize(st));
     stats->proposals = (int64_t)h.proposals;
     stats->screened_out = (int64_t)h.screened_out;
