@@ -79,6 +79,8 @@ __device__ inline int64_t lower_bound_i(const int* __restrict__ key, int64_t lo,
 enum { DN_NONE = 0, DN_REAL = 1, DN_COMPLEX = 2 };   // DN_NONE: line by line (opacity_kernel)
 struct DensePlan {
   int kind, m1, mh, m2;
+  float ih;                 // moments are of lengths times ih (a power of two)
+  int lines;                // divided blocks line by line, not by their groups' moments
 };
 
 // Whether a species' list is dense enough on this grid for those kernels;

@@ -24,6 +24,9 @@
 // first term left out is then below 9 DN_RHO^8 = 1.3e-6 of a line's own at the
 // nearest point for the line farthest from the centre, far below that in a sum.
 //
+// Lengths are in units of a power of two near the widest profile, so that no
+// power of a width leaves the FP32 range.
+//
 // Lorentz widths beyond about 3 points need moments about a complex centre:
 // with the lines of a block in bins of gamma_ref (ratio <= sqrt 2 within a bin),
 // u = delta + g + i (gamma - gamma_c) about the bin's middle gamma_c and
@@ -49,14 +52,18 @@
 // per point, where blocks pay for their fixed cost, and for cells whose widths
 // fit: Doppler widths that keep |x| >= 9 from the first mid block on; Lorentz
 // widths up to about 3 grid points, or gamma_ref within a factor 4 over the
-// list (4 bins) and widths below a sixth of the cutoff (the moments of the
-// divided blocks are about the real centre), or a cutoff so short that the near
-// window holds all of it.  Other cells go line by line.
+// list (4 bins), or a cutoff so short that the near window holds all of it.
+// Other cells go line by line.  From a sixth of the cutoff on a divided block's
+// moments about the real centre do not converge, and its lines count one by one
+// (130 of them per point; line by line the cell has 42,000).
 // Measured: one species of the 5e6-line grid (1.67e6 lines, 100,000 points), 10
 // layers over 1e-8 .. 100 bar x 20 temperatures: 169 ms line by line, 58 ms with
-// the 160 cells of widths up to 3 points here, 44 ms with the wider ones too;
+// the 160 cells of widths up to 3 points here, 44 ms with widths up to a sixth of
+// the cutoff, 40 ms with the near points in packed pairs, 28 ms with all cells
+// (100 us of the near kernel and 15 of the sums per Doppler cell, whose near
+// points' profiles bound it: 80% of the issue slots);
 // 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart: 2.59 ms and
-// 0.33 ms.
+// 0.31 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -86,6 +93,7 @@ constexpr size_t DN_SCRATCH = (size_t)256 << 20;     // moments and windows of a
 struct DensePoint {           // per grid point (indexes of groups and blocks)
   int gl, gr;                 // groups whose window holds the point: [gl, gr)
   int bl, br;                 // blocks all of whose lines do: [bl, br)
+  int il, ir;                 // lines: [il, ir)
 };
 
 // Lines whose window is not empty: [r[0], r[1]).
@@ -198,6 +206,8 @@ __global__ void dense_point_kernel(const LineWin* __restrict__ win, const int* _
   p.br = ir < i1 ? block_of(win[ir].jc, boff) : nb;
   p.bl = min(max(p.bl, 0), nb);             // in range for a list that is not sorted, too
   p.br = min(max(p.br, 0), nb);
+  p.il = il;
+  p.ir = ir;
   pts[j] = p;
 }
 
@@ -256,17 +266,17 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
   const DenseBins bn = dense_bins(stat);
   if (c == 0) *bins = bn;
   if (c >= n_cells) return;
-  DensePlan p{DN_NONE, 0, 0, 0};
+  DensePlan p{DN_NONE, 0, 0, 0, 1.0f, 0};
   const float scale = cells[c].gfac * inv_dnu, g = __int_as_float(stat[0]) * scale;   // widest line, in points
   if (cells[c].dense && !stat[1] && g < 1e6f) {
     // a point of block t is at least 8 m - 3.5 points from the centre of block t +- m
     const int m1 = max(DN_M1, (int)ceilf((sqrtf(16.0f + g * g) / DN_RHO + 3.5f) / 8.0f));
     const int m2 = max(4, (int)ceilf((sqrtf(256.0f + g * g) / DN_RHO + 15.5f) / 32.0f));
     if (m1 <= DN_M1_MAX) {
-      p = {DN_REAL, m1, 0, m2};
+      p = {DN_REAL, m1, 0, m2, 1.0f, 0};
     } else if (8 * (DN_M1_MAX - 1) > reach) {    // the near window holds every line's points
-      p = {DN_REAL, DN_M1_MAX, 0, m2};
-    } else if (bn.n > 0 && sqrtf(16.0f + g * g) <= DN_RHO_EDGE * (float)(reach - 8)) {
+      p = {DN_REAL, DN_M1_MAX, 0, m2, 1.0f, 0};
+    } else if (bn.n > 0) {
       float d8 = 0.0f, d32 = 0.0f;               // squared distances from which the complex moments hold
       for (int q = 0; q < bn.n; ++q) {
         const float gc = bn.c[q] * scale, e2 = bn.eta * bn.eta * gc * gc;
@@ -277,87 +287,124 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
       p.m1 = d8 > 0.0f ? (int)ceilf((sqrtf(d8) + 3.5f) / 8.0f) : 0;
       p.mh = d32 > 0.0f ? (int)ceilf((sqrtf(d32) + 15.5f) / 32.0f) : 0;
       p.m2 = max(m2, p.mh);
+      // the moments of the divided blocks' groups are about the real centre
+      p.lines = sqrtf(16.0f + g * g) > DN_RHO_EDGE * (float)(reach - 8);
     }
+    // lengths up to sqrt(16^2 + g^2): their 14th powers times a strength stay in range
+    p.ih = exp2f(-ceilf(0.5f * log2f(256.0f + g * g)));
   }
   plan[c] = p;
 }
 
-// G(x) = -Im w'(x) = (2 / sqrt(pi)) (2 x F(x) - 1), F Dawson's integral, x >= 0:
-// up to 9.3 a rational function of x^2 fitted (least squares, reweighted
+// Pairs of points in packed FP32 (one issue slot for both; the near kernel is
+// bound by issue).
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 rcp2(float2 d) { return make_float2(bartw::rcp_approx(d.x), bartw::rcp_approx(d.y)); }
+
+// G(x) = -Im w'(x) = (2 / sqrt(pi)) (2 x F(x) - 1), F Dawson's integral, u = x^2:
+// up to x = 9.3 a rational function of u fitted (least squares, reweighted
 // towards the largest error) to |dG| <= 1e-6 (50 e^(-x^2) + |G|) in FP32 -- near
 // its zero at 0.92 the Gaussian term of the profile is far larger -- and its
 // asymptotic series beyond.
-__device__ __forceinline__ float dawson_g(float x, float u) {
-  float n = 4.43394788e-06f, d = 7.85838861e-06f;
-  n = fmaf(n, u, -3.46022744e-05f);
-  n = fmaf(n, u, 4.63677612e-04f);
-  n = fmaf(n, u, -2.12909611e-04f);
-  n = fmaf(n, u, 2.23139278e-02f);
-  n = fmaf(n, u, -9.76259707e-02f);
-  n = fmaf(n, u, 1.38819137f);
-  n = fmaf(n, u, -1.12835006f);
-  d = fmaf(d, u, -7.29758443e-05f);
-  d = fmaf(d, u, 8.88062378e-04f);
-  d = fmaf(d, u, -8.60452054e-04f);
-  d = fmaf(d, u, 1.95862562e-02f);
-  d = fmaf(d, u, 6.41052559e-02f);
-  d = fmaf(d, u, 2.97722797e-01f);
-  d = fmaf(d, u, 7.68709942e-01f);
-  d = fmaf(d, u, 1.0f);
-  const bool far = x > 9.3f;
-  const float t = bartw::rcp_approx(far ? u : d);
-  float s = fmaf(t, 29.53125f, 6.5625f);       // (2k-1)!! / 2^k, k = 5 .. 1
-  s = fmaf(s, t, 1.875f);
-  s = fmaf(s, t, 0.75f);
-  s = fmaf(s, t, 0.5f);
-  return t * (far ? 1.1283791670955126f * s : n);
+__device__ __forceinline__ float2 dawson_g(float2 u) {
+  float2 n = f2(4.43394788e-06f), d = f2(7.85838861e-06f);
+  n = fma2(n, u, f2(-3.46022744e-05f));
+  n = fma2(n, u, f2(4.63677612e-04f));
+  n = fma2(n, u, f2(-2.12909611e-04f));
+  n = fma2(n, u, f2(2.23139278e-02f));
+  n = fma2(n, u, f2(-9.76259707e-02f));
+  n = fma2(n, u, f2(1.38819137f));
+  n = fma2(n, u, f2(-1.12835006f));
+  d = fma2(d, u, f2(-7.29758443e-05f));
+  d = fma2(d, u, f2(8.88062378e-04f));
+  d = fma2(d, u, f2(-8.60452054e-04f));
+  d = fma2(d, u, f2(1.95862562e-02f));
+  d = fma2(d, u, f2(6.41052559e-02f));
+  d = fma2(d, u, f2(2.97722797e-01f));
+  d = fma2(d, u, f2(7.68709942e-01f));
+  d = fma2(d, u, f2(1.0f));
+  const bool fx = u.x > 9.3f * 9.3f, fy = u.y > 9.3f * 9.3f;
+  const float2 t = rcp2(make_float2(fx ? u.x : d.x, fy ? u.y : d.y));
+  constexpr float C = 1.1283791670955126f;
+  float2 s = fma2(t, f2(29.53125f * C), f2(6.5625f * C));    // (2 / sqrt(pi)) (2k-1)!! / 2^k, k = 5 .. 1
+  s = fma2(s, t, f2(1.875f * C));
+  s = fma2(s, t, f2(0.75f * C));
+  s = fma2(s, t, f2(0.5f * C));
+  return mul2(t, make_float2(fx ? s.x : n.x, fy ? s.y : n.y));
 }
 
 // Re w(x + i y) for 0 <= y <= SMALL_Y: the expansion in y of small_y_re
 // (faddeeva.cuh) without a branch or a table.
-__device__ __forceinline__ float core_small(float x, float y) {
+__device__ __forceinline__ float2 core_small(float2 x, float y) {
   constexpr float L2E_LO = (float)(1.4426950408889634 - (double)LOG2EF);
-  const float u = x * x, lo = fmaf(x, x, -u);          // x^2 = u + lo
-  const float ah = -u * LOG2EF;
-  const float al = -fmaf(u, LOG2EF, ah) - fmaf(lo, LOG2EF, u * L2E_LO);
-  const float e = ex2f_approx(ah) * fmaf(al, LN2F_, 1.0f);
-  const float g = dawson_g(x, u);
-  const float y2 = y * y;
-  const float cub = x < 40.0f ? fmaf(g, fmaf(-4.0f, u, 6.0f), 2.2567583341910252f) : 0.0f;
-  return fmaf(e, fmaf(y2, fmaf(-2.0f, u, 1.0f), 1.0f), y * fmaf(y2 * (1.0f / 6.0f), cub, g));
+  const float2 u = mul2(x, x), lo = fma2(x, x, make_float2(-u.x, -u.y));     // x^2 = u + lo
+  const float2 ah = mul2(u, f2(-LOG2EF));
+  const float2 al = add2(fma2(u, f2(LOG2EF), ah), fma2(lo, f2(LOG2EF), mul2(u, f2(L2E_LO))));
+  const float2 e = mul2(make_float2(ex2f_approx(ah.x), ex2f_approx(ah.y)), fma2(al, f2(-LN2F_), f2(1.0f)));
+  const float2 g = dawson_g(u);
+  const float y2 = y * y, y26 = y2 * (1.0f / 6.0f);
+  const float2 q = make_float2(u.x < 1600.0f ? y26 : 0.0f, u.y < 1600.0f ? y26 : 0.0f);
+  const float2 gy = fma2(q, fma2(g, fma2(u, f2(-4.0f), f2(6.0f)), f2(2.2567583341910252f)), g);
+  return fma2(e, fma2(f2(y2), fma2(u, f2(-2.0f), f2(1.0f)), f2(1.0f)), mul2(f2(y), gy));
 }
 
 // (sqrt(pi) / y) Re w by Gauss-Hermite quadrature of w = (i / pi) int e^(-t^2) /
 // (z - t) dt: Re w = (y / pi) sum_k w_k / ((x - t_k)^2 + y^2), the two nodes +-t
 // as 2 w s / (s^2 - 4 x^2 t^2) with s = x^2 + y^2 + t^2.  Weights divided by
-// sqrt(pi) here.  4 nodes: <= 3.6e-7 for |z| >= 9.
-__device__ __forceinline__ float gh4_ratio(float x, float y2) {
+// sqrt(pi) here.  4 nodes: <= 4e-7 from |x| = gh4_from(y) on.
+__device__ __forceinline__ float2 gh4_ratio(float2 x, float y2) {
   constexpr float T1 = 0.27525512860841095f, T2 = 2.7247448713915889f;      // t^2
   constexpr float W1 = 0.90824829046386302f, W2 = 0.091751709536136983f;    // 2 w / sqrt(pi)
-  const float u = x * x, s1 = u + (y2 + T1), s2 = u + (y2 + T2);
-  const float d1 = fmaf(s1, s1, -4.0f * T1 * u), d2 = fmaf(s2, s2, -4.0f * T2 * u);
-  const float n = fmaf(W2 * s2, d1, W1 * s1 * d2);
-  return n * bartw::rcp_approx(d1 * d2);
+  const float2 u = mul2(x, x), s1 = add2(u, f2(y2 + T1)), s2 = add2(u, f2(y2 + T2));
+  const float2 d1 = fma2(s1, s1, mul2(u, f2(-4.0f * T1))), d2 = fma2(s2, s2, mul2(u, f2(-4.0f * T2)));
+  const float2 n = fma2(mul2(s2, f2(W2)), d1, mul2(mul2(s1, f2(W1)), d2));
+  return mul2(n, rcp2(mul2(d1, d2)));
 }
-// 8 nodes: <= 1.5e-7 for |z| >= 5, plus the residue e^(y^2 - x^2) cos 2xy that
-// the quadrature misses near the real axis.
-__device__ __forceinline__ float gh8_re(float x, float y) {
+// |x| from which it holds for widths of at least y; negative: everywhere.
+__device__ __forceinline__ float gh4_from(float y) { return y >= 7.0f ? -1.0f : y >= 4.0f ? 5.0f : y >= 2.0f ? 7.1f : 9.0f; }
+// 8 nodes: <= 3e-7 for |z| >= 5 and for y >= 3, plus the residue e^(y^2 - x^2)
+// cos 2xy that the quadrature misses near the real axis.
+constexpr float GH8_Y = 3.0f;
+constexpr float LORENTZ_Y = 1000.0f;        // from here on the shifted Lorentz form holds at any x (2 / y^2), and
+                                            // not much farther the products of the others leave the FP32 range
+template <bool RESIDUE>
+__device__ __forceinline__ float2 gh8_re(float2 x, float y) {
   constexpr float T[4] = {0.14530352150331707f, 1.3390972881263614f, 3.9269635013582872f, 8.5886356890120343f};
   constexpr float Wt[4] = {0.746024515358155f, 0.234479815323518f, 0.0192704402415765f, 0.00022522907675073f};
-  const float u = x * x, y2 = y * y;
-  float r = 0.0f;
+  const float y2 = y * y;
+  const float2 u = mul2(x, x);
+  float2 r = f2(0.0f);
 #pragma unroll
   for (int k = 0; k < 4; k += 2) {
-    const float s1 = u + (y2 + T[k]), s2 = u + (y2 + T[k + 1]);
-    const float d1 = fmaf(s1, s1, -4.0f * T[k] * u), d2 = fmaf(s2, s2, -4.0f * T[k + 1] * u);
-    r = fmaf(fmaf(Wt[k + 1] * s2, d1, Wt[k] * s1 * d2), bartw::rcp_approx(d1 * d2), r);
+    const float2 s1 = add2(u, f2(y2 + T[k])), s2 = add2(u, f2(y2 + T[k + 1]));
+    const float2 d1 = fma2(s1, s1, mul2(u, f2(-4.0f * T[k]))), d2 = fma2(s2, s2, mul2(u, f2(-4.0f * T[k + 1])));
+    r = fma2(fma2(mul2(s2, f2(Wt[k + 1])), d1, mul2(mul2(s1, f2(Wt[k])), d2)), rcp2(mul2(d1, d2)), r);
   }
-  const float g = fmaf(y, y, -u);
-  const float e = (y < 1.0f && g > -87.0f) ? __expf(g) * __cosf(2.0f * x * y) : 0.0f;
-  return fmaf(bartw::INV_SQRTPI * y, r, e);
+  r = mul2(r, f2(bartw::INV_SQRTPI * y));
+  if (RESIDUE) {
+    const float gx = fmaf(y, y, -u.x), gy = fmaf(y, y, -u.y);
+    if (y < 1.0f && gx > -87.0f) r.x += __expf(gx) * __cosf(2.0f * x.x * y);
+    if (y < 1.0f && gy > -87.0f) r.y += __expf(gy) * __cosf(2.0f * x.y * y);
+  }
+  return r;
 }
-__device__ __forceinline__ float core_any(float x, float y, const float2* __restrict__ wtab) {
-  return fmaf(x, x, y * y) < 25.0f ? bartw::taylor_re<1>(x, y, wtab) : gh8_re(x, y);
+// (sqrt(pi) / y) Re w for |z| >= 9: three terms of the asymptotic series from
+// |z| = 100 on (4e-8), else four nodes.
+__device__ __forceinline__ float far_ratio(float x, float y2) {
+  const float u = x * x, s = u + y2, r = bartw::rcp_approx(s);
+  if (s >= 1e4f) return r * fmaf(r * r, fmaf(1.5f, u, -0.5f * y2), 1.0f);
+  return gh4_ratio(f2(x), y2).x;
+}
+__device__ __forceinline__ float2 core_any(float2 x, float y, const float2* __restrict__ wtab) {
+  const bool tx = fmaf(x.x, x.x, y * y) < 25.0f, ty = fmaf(x.y, x.y, y * y) < 25.0f;
+  float2 r = f2(0.0f);
+  if (!tx || !ty) r = gh8_re<true>(x, y);
+  if (tx) r.x = bartw::taylor_re<>(fabsf(x.x), y, wtab);
+  if (ty) r.y = bartw::taylor_re<>(fabsf(x.y), y, wtab);
+  return r;
 }
 
 struct DenseArgs {
@@ -388,6 +435,7 @@ struct DenseArgs {
 struct NearShared {
   float4 acc[DN_WARPS][DN_WIN / 4][32];      // per lane, four neighbouring points
   float group[DN_WARPS][DN_GROUPS][DN_P];
+  int list[DN_WARPS][64];                    // lines of a bin, being gathered
 };
 
 __global__ void __launch_bounds__(32 * DN_WARPS)
@@ -450,10 +498,10 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     const float dx = a.dnu * inv, xc = w.delta * inv;
     const float off = (float)(w.jc - w0);                     // the line's nearest point in the window (exact)
 
-    // ---- moments about the block's centre, in points
+    // ---- moments about the block's centre, in points (times ih)
     {
-      const float de = (off - centre) - w.delta * a.inv_dnu, ga = gam * a.inv_dnu;
-      const float rdx = bartw::rcp_approx(dx), s2 = 0.5f * rdx * rdx;
+      const float de = ((off - centre) - w.delta * a.inv_dnu) * plan.ih, ga = gam * (a.inv_dnu * plan.ih);
+      const float rdx = bartw::rcp_approx(dx) * plan.ih, s2 = 0.5f * rdx * rdx;
       const float wt = S * a.w_scale;
       float M[DN_P];
       float r0 = 1.0f, i0 = 0.0f, r1 = de, i1 = ga;
@@ -502,47 +550,64 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     const float ymin = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(y)));
     const bool small = ymax <= bartw::SMALL_Y;
     // |x| from which the shifted Lorentz form holds for every lane
+    const bool lorentz = ymin >= LORENTZ_Y;
     const float xl = sqrtf(sqrtf(fmaf(2.0f * ymax, ymax, 1.5f) * (1.0f / DN_EPS_L)) * 1.001f);
-    const float x_core = ymin >= 9.0f ? -1.0f : 9.0f;         // |z| >= 9 everywhere: no core
+    const float x_core = gh4_from(ymin);
     const float rdm = bartw::rcp_approx(dxm);
     const float p_far = xl * rdm, p_core = x_core * rdm;      // the same distances in points
-    const float qL = q - 1.5f;
+    const float p_tab = 5.0f * rdm;                           // |z| >= 5: no table
+    const float2 qL = f2(q - 1.5f), dx2 = f2(dx), xc2 = f2(xc);
     const int jl = w.jlo - w0, jh = w.jhi - w0;
-    for (int s = 0; s < steps; ++s) {
-      const float p0 = (float)(4 * s);
-      const float gap = fmaxf(cmin - (p0 + 3.0f), p0 - cmax);   // distance of the four points from the lines
-      const float k0 = p0 - off;
-      float v[4];
-      if (gap >= p_far) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float x = fmaf(k0 + (float)k, dx, xc);
-          v[k] = A * bartw::rcp_approx(fmaf(x, x, qL));
-        }
-      } else if (gap >= p_core) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = A * gh4_ratio(fmaf(k0 + (float)k, dx, xc), q);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float p = p0 + (float)k;
-          const float x = fabsf(fmaf(k0 + (float)k, dx, xc));
-          if (fmaxf(cmin - p, p - cmax) >= p_core) v[k] = A * gh4_ratio(x, q);
-          else if (small) v[k] = B * core_small(x, y);
-          else v[k] = B * core_any(x, y, a.wtab);
-        }
-      }
-      if (check) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (4 * s + k < jl || 4 * s + k > jh) v[k] = 0.0f;
-      }
+    // steps of four points [0, s1) and [s4, steps) are far from every line,
+    // [s1, s2) and [s3, s4) beyond the core, [s2, s3) within it for some
+    auto left = [&](float d) { return min(max((int)floorf((cmin - d + 1.0f) * 0.25f), 0), steps); };
+    auto right = [&](float d, int from) { return min(max((int)ceilf((cmax + d) * 0.25f), from), steps); };
+    const int s1 = lorentz ? steps : left(p_far), s2 = max(left(p_core), s1);
+    const int s3 = x_core < 0.0f ? s2 : right(p_core, s2), s4 = right(p_far, s3);
+    auto add = [&](int s, float A0, float2 r0, float2 r1) {   // acc += A0 r
       float4 t = acc[s][lane];
-      t.x += v[0];
-      t.y += v[1];
-      t.z += v[2];
-      t.w += v[3];
+      if (check) {                                            // (an infinite A0 stays within the line's window)
+        const float2 v0 = mul2(f2(A0), r0), v1 = mul2(f2(A0), r1);
+        const int j = 4 * s;
+        if (j >= jl && j <= jh) t.x += v0.x;
+        if (j + 1 >= jl && j + 1 <= jh) t.y += v0.y;
+        if (j + 2 >= jl && j + 2 <= jh) t.z += v1.x;
+        if (j + 3 >= jl && j + 3 <= jh) t.w += v1.y;
+      } else {
+        const float2 t0 = fma2(f2(A0), r0, make_float2(t.x, t.y)), t1 = fma2(f2(A0), r1, make_float2(t.z, t.w));
+        t = make_float4(t0.x, t0.y, t1.x, t1.y);
+      }
       acc[s][lane] = t;
+    };
+    auto at = [&](int s, int k) {                             // x of points 4 s + k and the next
+      const float k0 = (float)(4 * s) - off;
+      return fma2(add2(f2(k0), make_float2((float)k, (float)(k + 1))), dx2, xc2);
+    };
+    for (int e = steps - s4 + s1; e > 0; --e) {
+      const int s = e > s1 ? steps - (e - s1) : s1 - e;
+      const float2 xa = at(s, 0), xb = at(s, 2);
+      add(s, A, rcp2(fma2(xa, xa, qL)), rcp2(fma2(xb, xb, qL)));
+    }
+    for (int e = (s2 - s1) + (s4 - s3); e > 0; --e) {
+      const int s = e > s2 - s1 ? s4 - (e - (s2 - s1)) : s2 - e;
+      add(s, A, gh4_ratio(at(s, 0), q), gh4_ratio(at(s, 2), q));
+    }
+    if (small) {
+      for (int s = s2; s < s3; ++s) add(s, B, core_small(at(s, 0), y), core_small(at(s, 2), y));
+    } else if (ymin >= GH8_Y) {
+      for (int s = s2; s < s3; ++s) add(s, B, gh8_re<false>(at(s, 0), y), gh8_re<false>(at(s, 2), y));
+    } else {
+      for (int s = s2; s < s3; ++s) {
+        const float p0 = (float)(4 * s);
+        float2 r[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float2 x = at(s, 2 * k);
+          const float p = p0 + (float)(2 * k);
+          r[k] = fmaxf(cmin - (p + 1.0f), p - cmax) >= p_tab ? gh8_re<true>(x, y) : core_any(x, y, a.wtab);
+        }
+        add(s, B, r[0], r[1]);
+      }
     }
     if (++chunks % DN_FOLD == 0 && base + 32 < l1) {
       fold();
@@ -563,36 +628,56 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     a.m8[at * DN_P + lane] = t;
   }
   if (plan.kind != DN_COMPLEX) return;
-  // ---- moments about the complex centres, a pass over the lines per bin
+  // ---- moments about the complex centres, bin by bin; the bin's lines are
+  // gathered in shared memory first, so that 32 of them are taken at a time
   const DenseBins bn = *a.bins;
+  int* list = sh.list[warp];
   for (int bin = 0; bin < bn.n; ++bin) {
     float2 M[DN_PC];
 #pragma unroll
     for (int n = 0; n < DN_PC; ++n) M[n] = make_float2(0.f, 0.f);
     const float gc = bn.c[bin] * cc.gfac;
+    int have = 0;
     for (int base = l0; base < l1; base += 32) {
-      const int i = min(base + lane, l1 - 1);
-      const LineWin w = a.win[i];
-      const float gr = a.gref[i];
-      const int mine = min(max((int)floorf(log2f(gr * bn.inv_g0) * bn.inv_lr), 0), bn.n - 1);
-      const float ln_s = line_ln_s(w, cc);
-      const bool take = base + lane < l1 && mine == bin && ln_s >= ln_thr;
-      const float wt = take ? ex2f_approx((ln_s + LN_SCALE) * LOG2EF) * a.w_scale : 0.0f;
-      const float inv = bartw::rcp_approx(w.nu0f * cc.dfac), rdx = bartw::rcp_approx(a.dnu * inv), s2 = 0.5f * rdx * rdx;
-      const float de = ((float)(w.jc - w0) - centre) - w.delta * a.inv_dnu, ga = (gr * cc.gfac - gc) * a.inv_dnu;
-      // K_0 = 1, K_1 = u, K_(n+1) = u K_n + n sigma^2 K_(n-1), weighted
-      float r0 = wt, i0 = 0.0f, r1 = de * wt, i1 = ga * wt;
+      const int next = base + lane;
+      const bool in = next < l1 &&
+                      min(max((int)floorf(log2f(a.gref[min(next, l1 - 1)] * bn.inv_g0) * bn.inv_lr), 0), bn.n - 1) == bin;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) list[have + __popc(m & ((1u << lane) - 1u))] = next;
+      have += __popc(m);
+      __syncwarp();
+      if (have < 32 && base + 32 < l1) continue;
+      do {                                       // 32 lines, or at the end what is left
+        const bool on = lane < have;
+        const int i = list[on ? lane : 0];
+        const LineWin w = a.win[have > 0 ? i : l0];
+        const float gr = a.gref[have > 0 ? i : l0];
+        const float ln_s = line_ln_s(w, cc);
+        const float wt = (on && ln_s >= ln_thr) ? ex2f_approx((ln_s + LN_SCALE) * LOG2EF) * a.w_scale : 0.0f;
+        const float inv = bartw::rcp_approx(w.nu0f * cc.dfac), rdx = bartw::rcp_approx(a.dnu * inv) * plan.ih, s2 = 0.5f * rdx * rdx;
+        const float de = (((float)(w.jc - w0) - centre) - w.delta * a.inv_dnu) * plan.ih;
+        const float ga = (gr * cc.gfac - gc) * (a.inv_dnu * plan.ih);
+        // K_0 = 1, K_1 = u, K_(n+1) = u K_n + n sigma^2 K_(n-1), weighted
+        float r0 = wt, i0 = 0.0f, r1 = de * wt, i1 = ga * wt;
 #pragma unroll
-      for (int n = 0; n < DN_PC; ++n) {
-        M[n].x += r0;
-        M[n].y += i0;
-        const float ns = (float)(n + 1) * s2;
-        const float r2 = fmaf(de, r1, fmaf(-ga, i1, ns * r0)), i2 = fmaf(de, i1, fmaf(ga, r1, ns * i0));
-        r0 = r1;
-        i0 = i1;
-        r1 = r2;
-        i1 = i2;
-      }
+        for (int n = 0; n < DN_PC; ++n) {
+          M[n].x += r0;
+          M[n].y += i0;
+          const float ns = (float)(n + 1) * s2;
+          const float r2 = fmaf(de, r1, fmaf(-ga, i1, ns * r0)), i2 = fmaf(de, i1, fmaf(ga, r1, ns * i0));
+          r0 = r1;
+          i0 = i1;
+          r1 = r2;
+          i1 = i2;
+        }
+        __syncwarp();
+        const int rest = list[32 + lane];        // those beyond the 32 taken, at most 31
+        __syncwarp();
+        list[lane] = rest;
+        __syncwarp();
+        have -= 32;
+      } while (have > 0 && base + 32 >= l1);
+      have = max(have, 0);
     }
     float2 mine = make_float2(0.f, 0.f);
 #pragma unroll
@@ -613,13 +698,13 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
 __global__ void __launch_bounds__(128)
 dense_up_kernel(const __grid_constant__ DenseArgs a) {
   const int P = blockIdx.x * blockDim.x + threadIdx.x;
-  const int kind = a.plan[a.c0 + blockIdx.y].kind;
-  if (P >= a.nb / 4 || kind == DN_NONE) return;
+  const DensePlan plan = a.plan[a.c0 + blockIdx.y];
+  if (P >= a.nb / 4 || plan.kind == DN_NONE) return;
   const float* m = a.m8 + ((int64_t)blockIdx.y * a.nb + 4 * P) * DN_P;
   float o[DN_P] = {};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const float t = (float)(8 * c - 12);
+    const float t = (float)(8 * c - 12) * plan.ih;
     float v[DN_P];
 #pragma unroll
     for (int n = 0; n < DN_P; ++n) v[n] = m[c * DN_P + n];
@@ -635,12 +720,12 @@ dense_up_kernel(const __grid_constant__ DenseArgs a) {
   float* d = a.m32 + ((int64_t)blockIdx.y * (a.nb / 4) + P) * DN_P;
 #pragma unroll
   for (int n = 0; n < DN_P; ++n) d[n] = o[n];
-  if (kind != DN_COMPLEX) return;
+  if (plan.kind != DN_COMPLEX) return;
   for (int bin = 0; bin < a.bins->n; ++bin) {
     float2 u[DN_PC] = {};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const float t = (float)(8 * c - 12);
+      const float t = (float)(8 * c - 12) * plan.ih;
       const float2* src = a.mc8 + (((int64_t)blockIdx.y * a.nb + 4 * P + c) * DN_BINS + bin) * DN_PC;
       float2 v[DN_PC];
 #pragma unroll
@@ -658,7 +743,7 @@ dense_up_kernel(const __grid_constant__ DenseArgs a) {
   }
 }
 
-// sum_n I_n / D^(n+1)
+// sum_n I_n / D^(n+1), D in the moments' unit (the sums are in it, too)
 __device__ __forceinline__ float moment_sum(const float* __restrict__ m, float D) {
   const float4 a = *reinterpret_cast<const float4*>(m), b = *reinterpret_cast<const float4*>(m + 4);
   const float r = bartw::rcp_approx(D);
@@ -708,10 +793,11 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   const float* m32 = a.m32 + (int64_t)blockIdx.y * (a.nb / 4) * DN_P;
   const float* mg = a.mg + (int64_t)blockIdx.y * a.g_stride * DN_P;
   const float* win = a.window + (int64_t)blockIdx.y * a.nb * DN_WIN;
-  const float jf = (float)(j - j0);                          // positions relative to j0: exact
-  // centre of block b and of parent P, relative to j0
-  auto centre8 = [&](int b) { return (float)((b - a.boff) * DN_B - j0) + 3.5f; };
-  auto centre32 = [&](int P) { return (float)((4 * P - a.boff) * DN_B - j0) + 15.5f; };
+  // distances from the centres of block b and parent P, in the moments' unit (exact)
+  const float e8 = ((float)(j & 7) - 3.5f) * plan.ih, f8 = -8.0f * plan.ih;
+  const float e32 = ((float)(j & 31) - 15.5f) * plan.ih, f32 = -32.0f * plan.ih;
+  auto dist8 = [&](int b) { return fmaf((float)(b - t), f8, e8); };
+  auto dist32 = [&](int P) { return fmaf((float)(P - T), f32, e32); };
 
   // ---- near: the windows of the blocks around the point
   float near = 0.0f;
@@ -723,7 +809,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   float far = 0.0f, mid = 0.0f;
   if (plan.kind == DN_COMPLEX) {
     const DenseBins bn = *a.bins;
-    const float scale = a.cells[cell].gfac * a.inv_dnu;
+    const float scale = a.cells[cell].gfac * a.inv_dnu * plan.ih;
     const float2* mc8 = a.mc8 + (int64_t)blockIdx.y * a.nb * DN_BINS * DN_PC;
     const float2* mc32 = a.mc32 + (int64_t)blockIdx.y * (a.nb / 4) * DN_BINS * DN_PC;
     // parents inside the cutoff: real centre far away, complex centres nearer
@@ -731,7 +817,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
     for (int P = u0; P < u1; ++P) {
       const int m = abs(P - T);                  // the same for the warp
       const bool in = P >= PL && P < PR;
-      const float D = jf - centre32(P);
+      const float D = dist32(P);
       if (m >= plan.m2) {
         if (in) far += moment_sum(m32 + (int64_t)P * DN_P, D);
       } else if (m >= plan.mh) {
@@ -745,7 +831,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
       const int v1 = __reduce_max_sync(0xffffffffu, b0 < b1 ? b1 : -0x7fffffff);
       for (int b = v0; b < v1; ++b) {
         const bool in = b >= b0 && b < b1 && abs(b - t) >= plan.m1;
-        const float D = jf - centre8(b);
+        const float D = dist8(b);
         for (int q = 0; q < bn.n; ++q)
           if (in) mid += complex_sum(mc8 + ((int64_t)b * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
       }
@@ -765,16 +851,16 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   {
     const int u0 = __reduce_min_sync(0xffffffffu, PL), u1 = __reduce_max_sync(0xffffffffu, PE);
     for (int P = u0; P < u1; ++P)
-      if (P >= PL && P < PE) far += moment_sum(m32 + (int64_t)P * DN_P, jf - centre32(P));
+      if (P >= PL && P < PE) far += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
     const int v0 = __reduce_min_sync(0xffffffffu, PS), v1 = __reduce_max_sync(0xffffffffu, PR);
     for (int P = v0; P < v1; ++P)
-      if (P >= PS && P < PR) far += moment_sum(m32 + (int64_t)P * DN_P, jf - centre32(P));
+      if (P >= PS && P < PR) far += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
   }
   auto blocks = [&](int b0, int b1) {                        // [b0, b1), possibly empty
     const int u0 = __reduce_min_sync(0xffffffffu, b0 < b1 ? b0 : 0x7fffffff);
     const int u1 = __reduce_max_sync(0xffffffffu, b0 < b1 ? b1 : -0x7fffffff);
     for (int b = u0; b < u1; ++b)
-      if (b >= b0 && b < b1) mid += moment_sum(m8 + (int64_t)b * DN_P, jf - centre8(b));
+      if (b >= b0 && b < b1) mid += moment_sum(m8 + (int64_t)b * DN_P, dist8(b));
   };
   const bool hasL = PE > PL, hasR = PR > PS;
   blocks(p.bl, hasL ? min(4 * PL, lend) : lend);
@@ -784,20 +870,46 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   }
 
   // ---- edges: the block that a cutoff edge divides, group by group (blocks
-  // within the near radius were taken line by line)
-  float edge = 0.0f;
-  auto groups = [&](int g0, int g1, int b) {
-    if (abs(b - t) < plan.m1) return;
-    const float D = jf - centre8(b);
-    for (int g = max(g0, 0); g < min(g1, (int)a.g_stride); ++g) edge += moment_sum(mg + (int64_t)g * DN_P, D);
-  };
-  if (p.bl > p.br) {                                         // both edges divide the same block
-    groups(p.gl, p.gr, p.br);
+  // within the near radius were taken line by line), or, where the profiles
+  // are too wide for their moments about the real centre, line by line: at
+  // least 23 points away, |x| > 9 (dense_applies), by the far form
+  float edge = 0.0f, direct = 0.0f;
+  const bool both = p.bl > p.br;                             // both edges divide the same block
+  if (plan.lines) {
+    const CellConst cc = a.cells[cell];
+    const float ln_thr = a.smax ? ordered_float(a.smax[a.tmap[cell]]) + a.ln_rel : -3.0e38f;
+    auto lines = [&](int i0, int i1, int b) {
+      if (abs(b - t) < plan.m1) return;
+      for (int i = i0; i < i1; ++i) {
+        const LineWin w = a.win[i];
+        const float ln_s = line_ln_s(w, cc);
+        if (!(ln_s >= ln_thr)) continue;
+        const float inv = bartw::rcp_approx(w.nu0f * cc.dfac), y = a.gref[i] * cc.gfac * inv;
+        const float S = ex2f_approx((ln_s + LN_SCALE) * LOG2EF);
+        const float x = fmaf((float)(j - w.jc), a.dnu * inv, w.delta * inv);
+        direct = fmaf(S * inv * bartw::INV_SQRTPI * (y * bartw::INV_SQRTPI), far_ratio(x, y * y), direct);
+      }
+    };
+    if (both) {
+      lines(p.il, p.ir, p.br);
+    } else {
+      if (p.bl > 0) lines(p.il, min(a.lstart[p.bl], p.ir), p.bl - 1);
+      if (p.br < a.nb) lines(max(a.lstart[p.br], p.il), p.ir, p.br);
+    }
   } else {
-    if (p.bl > 0) groups(p.gl, min(a.gfirst[p.bl], p.gr), p.bl - 1);
-    if (p.br < a.nb) groups(max(a.gfirst[p.br], p.gl), p.gr, p.br);
+    auto groups = [&](int g0, int g1, int b) {
+      if (abs(b - t) < plan.m1) return;
+      const float D = dist8(b);
+      for (int g = max(g0, 0); g < min(g1, (int)a.g_stride); ++g) edge += moment_sum(mg + (int64_t)g * DN_P, D);
+    };
+    if (both) {
+      groups(p.gl, p.gr, p.br);
+    } else {
+      if (p.bl > 0) groups(p.gl, min(a.gfirst[p.bl], p.gr), p.bl - 1);
+      if (p.br < a.nb) groups(max(a.gfirst[p.br], p.gl), p.gr, p.br);
+    }
   }
-  if (j0 + lane < a.n_nu) a.out[(int64_t)cell * a.n_nu + j] = ((edge + far) + (mid + near)) * INV_SCALE;
+  if (j0 + lane < a.n_nu) a.out[(int64_t)cell * a.n_nu + j] = (((edge + far) + mid) * plan.ih + (near + direct)) * INV_SCALE;
 }
 
 }  // namespace

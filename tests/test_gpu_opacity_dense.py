@@ -126,3 +126,26 @@ def test_a_strong_line_that_has_been_cut_off_leaves_nothing(ctx):
         assert half.n < 0.5 * N
         ref += ctx.opacity_cells([bart.device_lines(half)], p, t, nu, 2.5).cpu().numpy()
     assert np.all(np.abs(got - ref) <= MAX_REL * ref + 3.0 * 2.0 ** -149)
+
+
+@pytest.mark.parametrize("dnu,cutoff,ratio", [(0.02, 25.0, 2.0), (0.02, 0.7, 1.0), (0.1, 25.0, 3.9), (1.0, 40.0, 1.3),
+                                              (0.005, 2.0, 3.0)])
+def test_profiles_wider_than_a_sixth_of_the_cutoff(ctx, dnu, cutoff, ratio):
+    """The lines of a block that a cutoff edge divides count one by one there;
+    strong lines, so that powers of the widths would leave the FP32 range."""
+    import paper_2104_12522_gb300 as bart
+    N = 300
+    lo, hi = 1000.0 - 1.2 * cutoff, 1000.0 + N * dnu + 1.2 * cutoff
+    ll = _list(0, int(1.5 * (hi - lo) / dnu), lo, hi, dnu, 11)
+    rng = np.random.default_rng(12)
+    ll = W.LineList(ll.nu0, ll.log10_s296 + 4.0, ll.elow, (0.1 * ratio ** -rng.uniform(0.0, 1.0, ll.n)).astype(np.float32),
+                    18.0)
+    g = np.array([0.2, 0.5, 3.0, 20.0]) * cutoff          # widths of the widest lines, cm^-1
+    t = np.array([600.0, 2500.0, 600.0, 1500.0])
+    p = g / 0.1 * np.sqrt(t / 296.0)
+    got = ctx.opacity_cells([bart.device_lines(ll)], p, t, bart.NuGrid(1000.0, dnu, N), cutoff)
+    ctx.sync()
+    ref = O.opacity_cells([ll], p, t, 1000.0, dnu, N, cutoff)
+    e, l2 = opacity_errors(got.cpu().numpy(), ref)
+    print(f"dnu {dnu} cutoff {cutoff}: max rel {e:.2e}, L2 {l2:.2e}")
+    assert e < MAX_REL and l2 < L2_REL
