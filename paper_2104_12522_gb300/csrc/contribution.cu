@@ -8,7 +8,10 @@
 //                        level integrated (kb: the deck, the optical-depth limit or
 //                        L-1) its blackbody seen through the column, and zeros
 //                        below.  sum_k C_k is the flux of the emission kernels.
-//   band_extent_kernel   first and last wavenumber at which each filter is not zero.
+//                        Its CTAs also find the first and last wavenumber at which
+//                        each filter is not zero, a proposal's CTAs taking every
+//                        n-th filter (a launch of their own for this and a memset
+//                        of its result were 5 of 53 us of one small spectrum).
 //   contrib_band_kernel  band means of the rows over those wavenumbers only.
 //
 // The pass reads 2 S grid rows per (proposal, layer) once and is bound by that
@@ -63,9 +66,24 @@ contrib_kernel(const float* __restrict__ grid, int L, int M, int64_t N, const La
                const float* __restrict__ coef, const float* __restrict__ dpg, const __grid_constant__ Angles ang,
                double nu_start, double dnu, const int64_t* __restrict__ nu_lo, const int64_t* __restrict__ nu_hi,
                float* __restrict__ contrib, const int32_t* __restrict__ act_mask, int* __restrict__ status,
-               EmExtra ex, int wide_x, int tau_lim, int* __restrict__ flag) {
+               EmExtra ex, int wide_x, int tau_lim, int* __restrict__ flag, const float* __restrict__ filt,
+               int n_bands, int* __restrict__ ext) {
   const int p = blockIdx.x;
   const int tid = threadIdx.x;
+  // ext[2 b] = N - first, ext[2 b + 1] = last + 1 over the wavenumbers where
+  // filter b is not zero (0, 0: none); ext starts at 0.  The CTAs along y
+  // cover the whole grid, whatever the spans are.
+  for (int b = p; b < n_bands; b += gridDim.x) {
+    const int64_t j = (int64_t)blockIdx.y * CF_TILE + 2 * tid;
+    const float* w = filt + (int64_t)b * N + j;
+    const bool on_a = j < N && __ldg(w) != 0.0f, on_b = j + 1 < N && __ldg(w + 1) != 0.0f;   // true for NaN
+    const int first = __reduce_max_sync(0xffffffffu, on_a ? (int)(N - j) : on_b ? (int)(N - j - 1) : 0);
+    const int last = __reduce_max_sync(0xffffffffu, on_b ? (int)(j + 2) : on_a ? (int)(j + 1) : 0);
+    if ((tid & 31) == 0 && last > 0) {
+      atomicMax(ext + 2 * b, first);
+      atomicMax(ext + 2 * b + 1, last);
+    }
+  }
   if (act_mask && !act_mask[p]) return;
   const int64_t lo = nu_lo ? nu_lo[p] : 0;
   const int64_t hi = nu_hi ? nu_hi[p] : N;
@@ -201,27 +219,6 @@ contrib_kernel(const float* __restrict__ grid, int L, int M, int64_t N, const La
   for (int q = k; q < L; ++q) store(q, f2(0.0f));
 }
 
-// ext[2 b] = N - first, ext[2 b + 1] = last + 1 over the wavenumbers where
-// filter b is not zero (0, 0: none); ext starts at 0.
-__global__ void __launch_bounds__(CB_THREADS)
-band_extent_kernel(const float* __restrict__ filt, int64_t N, int64_t per, int* __restrict__ ext) {
-  const int b = blockIdx.y;
-  const int64_t j0 = blockIdx.x * per, j1 = min(N, j0 + per);
-  int first = 0, last = 0;
-  for (int64_t j = j0 + threadIdx.x; j < j1; j += CB_THREADS) {
-    if (__ldg(filt + (int64_t)b * N + j) != 0.0f) {     // true for NaN
-      first = max(first, (int)(N - j));
-      last = max(last, (int)(j + 1));
-    }
-  }
-  first = __reduce_max_sync(0xffffffffu, first);
-  last = __reduce_max_sync(0xffffffffu, last);
-  if ((threadIdx.x & 31) == 0 && last > 0) {
-    atomicMax(ext + 2 * b, first);
-    atomicMax(ext + 2 * b + 1, last);
-  }
-}
-
 // Band means of CB_ROWS contribution rows of one proposal: trapezoid weights
 // over the proposal's span, the sums as FP32 pairs per thread and across the
 // warp, FP64 across the warps.
@@ -281,15 +278,15 @@ contrib_band_kernel(const float* __restrict__ contrib, int L, int64_t N, const i
 
 using CfLauncher = void (*)(dim3, cudaStream_t, const float*, int, int, int64_t, const LayerTW*, const float*,
                             const float*, const Angles&, double, double, const int64_t*, const int64_t*, float*,
-                            const int32_t*, int*, EmExtra, int, int, int*);
+                            const int32_t*, int*, EmExtra, int, int, int*, const float*, int, int*);
 
 template <int S, int NA>
 void launch_contrib(dim3 g, cudaStream_t st, const float* grid, int L, int M, int64_t N, const LayerTW* tw,
                     const float* coef, const float* dpg, const Angles& ang, double nu_start, double dnu,
                     const int64_t* lo, const int64_t* hi, float* contrib, const int32_t* active, int* status,
-                    EmExtra ex, int wide_x, int tau_lim, int* flag) {
+                    EmExtra ex, int wide_x, int tau_lim, int* flag, const float* filt, int n_bands, int* ext) {
   contrib_kernel<S, NA><<<g, CF_THREADS, 0, st>>>(grid, L, M, N, tw, coef, dpg, ang, nu_start, dnu, lo, hi, contrib,
-                                                  active, status, ex, wide_x, tau_lim, flag);
+                                                  active, status, ex, wide_x, tau_lim, flag, filt, n_bands, ext);
 }
 
 template <int S>
@@ -336,25 +333,25 @@ extern "C" bart_status bart_contribution_functions(bart_ctx* ctx, const bart_gri
   const int64_t N = g->nu.n_nu;
   BART_REQUIRE(ctx, (int64_t)n * L <= 2147483647LL, "n x n_layers too large");
   BART_CUDA(ctx, cudaSetDevice(ctx->device));
-  EmPrep pr;
-  if ((st = emission_prologue(ctx, g, c, b, &pr)) != BART_OK) return st;
   float* out = contrib;
   if (!out) {
     void* p = nullptr;
     if ((st = bart_scratch(ctx, "cf_rows", (size_t)n * L * N * sizeof(float), &p)) != BART_OK) return st;
     out = (float*)p;
   }
-  // band extents and the rows' flags, both starting at 0
+  // band extents and the rows' flags, both cleared by the prologue's launch
   int *ext = nullptr, *flag = nullptr;
+  size_t words = 0;
   std::vector<void*> held;
   if (nb > 0) {
-    const size_t words = 2 * (size_t)nb + (size_t)n * L;
+    words = 2 * (size_t)nb + (size_t)n * L;
     if ((st = bart_scratch_any(ctx, "cf_ext", words * sizeof(int), (void**)&ext, &held)) != BART_OK) return st;
     flag = ext + 2 * nb;
-    BART_CUDA(ctx, cudaMemsetAsync(ext, 0, words * sizeof(int), ctx->stream));
-    const int64_t per = std::max<int64_t>(4 * CB_THREADS, (N + 63) / 64);
-    band_extent_kernel<<<dim3((unsigned)((N + per - 1) / per), (unsigned)nb), CB_THREADS, 0, ctx->stream>>>(
-        f->weights, N, per, ext);
+  }
+  EmPrep pr;
+  if ((st = emission_prologue(ctx, g, c, b, &pr, ext, words)) != BART_OK) {
+    bart_scratch_give_back(ctx, &held);
+    return st;
   }
   const int mode = emission_mode(g, c);
   std::vector<double> mu, w;
@@ -367,7 +364,7 @@ extern "C" bart_status bart_contribution_functions(bart_ctx* ctx, const bart_gri
   const int64_t n_tiles = (N + 1 + CF_TILE - 1) / CF_TILE;     // an odd span start takes one pair more
   launch(dim3((unsigned)n, (unsigned)n_tiles), ctx->stream, g->grid, L, M, N, pr.tw, pr.coef, pr.dc + pr.off_dpg,
          ang, g->nu.nu_start_cm, g->nu.dnu_cm, b->nu_lo, b->nu_hi, out, b->active, ctx->d_status,
-         emission_extra(g, c), mode & 1, (mode >> 1) & 1, flag);
+         emission_extra(g, c), mode & 1, (mode >> 1) & 1, flag, nb > 0 ? f->weights : nullptr, nb, ext);
   st = bart_check_launch(ctx, "contrib_kernel");
   if (st == BART_OK && nb > 0) {
     const int64_t groups = (L + CB_ROWS - 1) / CB_ROWS;

@@ -102,7 +102,8 @@ inline bool fused_offsets_fit(const bart_grid_desc* g) {
 bart_status check_forward_request(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b);
 
 // Constants, layer brackets and abundance coefficients of an emission batch:
-// uploads the constant table and launches tp_kernel on the context's stream.
+// uploads the constant table and launches tp_kernel on the context's stream,
+// which also clears zero_words words at zero (later kernels' counters).
 struct EmPrep {
   const float* dc;      // [p_cgs L][t_axis M][dpg L-1][ang 2NA][x0 S]
   size_t off_dpg, off_ang;
@@ -110,7 +111,7 @@ struct EmPrep {
   float* coef;
 };
 bart_status emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
-                              EmPrep* out);
+                              EmPrep* out, int* zero = nullptr, size_t zero_words = 0);
 
 // The persistent fused launch of an emission batch (forward_fused.cu).
 bart_status fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,

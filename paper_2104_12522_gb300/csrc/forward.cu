@@ -40,8 +40,9 @@ __global__ void tp_kernel(const float* __restrict__ theta, int n_theta, const fl
                           int M, int64_t N, float inv_g, float tint4, float tirr0, float t_min, float t_max,
                           const float* __restrict__ x0_over_mu, LayerTW* __restrict__ tw,
                           float* __restrict__ coef, const int32_t* __restrict__ act_mask,
-                          int* __restrict__ status) {
+                          int* __restrict__ status, int* __restrict__ zero = nullptr, size_t zero_words = 0) {
   const int p = blockIdx.x;
+  for (size_t i = (size_t)p * blockDim.x + threadIdx.x; i < zero_words; i += (size_t)gridDim.x * blockDim.x) zero[i] = 0;
   if (p >= n) return;
   if (act_mask && !act_mask[p]) return;      // skipped entry (its parameters may lie outside the prior)
   for (int k = threadIdx.x; k < L; k += blockDim.x) {
@@ -415,7 +416,7 @@ bart_status bartem::check_forward_request(bart_ctx* ctx, const bart_grid_desc* g
 }
 
 bart_status bartem::emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
-                              EmPrep* out) {
+                              EmPrep* out, int* zero, size_t zero_words) {
   const int S = g->n_species, L = g->n_layers, M = g->n_temps, n = b->n;
   const int64_t N = g->nu.n_nu;
   std::vector<double> mu, w;
@@ -443,7 +444,7 @@ bart_status bartem::emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, co
   tp_kernel<<<n, 128, 0, ctx->stream>>>(b->theta, 5 + S, b->t_profile, n, L, S, dc, dc + off_t, M, N,
                                         (float)(1.0 / c->g_cgs), tint4, tirr0, (float)c->t_min_K,
                                         (float)std::min(c->t_max_K, 1e30), dc + off_x0, (LayerTW*)p_tw,
-                                        (float*)p_coef, b->active, ctx->d_status);
+                                        (float*)p_coef, b->active, ctx->d_status, zero, zero_words);
   if ((st = bart_check_launch(ctx, "tp_kernel")) != BART_OK) return st;
   out->dc = dc;
   out->off_dpg = off_dpg;
