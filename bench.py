@@ -49,10 +49,12 @@ N_ANGLES = 8
 N_BANDS = 10
 FW_SPECIES = 4                    # species of the forward-model generation's grid
 OPACITY_LAUNCHES_PER_STEP = 3     # one opacity kernel launch per species
-KERNELS_PER_STEP = 3 * 3 + 1      # per species: window and span prologues + opacity; one fused generation
+# per species: window and span prologues, nine of the dense list's, its three kernels (counted once: they repeat
+# per batch of cells that fits the scratch), the line-by-line kernel for the other cells; one fused generation
+KERNELS_PER_STEP = 3 * (2 + 9 + 3 + 1) + 1
 # sources the opacity kernel is compiled from (the committed traffic figure is tied to them)
 OPACITY_SOURCES = [os.path.join(ROOT, "paper_2104_12522_gb300", "csrc", f)
-                   for f in ("opacity.cu", "faddeeva.cuh", "bart_internal.cuh")]
+                   for f in ("opacity.cu", "opacity_dense.cu", "opacity.cuh", "faddeeva.cuh", "bart_internal.cuh")]
 FORWARD_SOURCES = [os.path.join(ROOT, "paper_2104_12522_gb300", "csrc", f)
                    for f in ("emission_fused.cuh", "forward_fused.cu", "emission.cuh", "forward.cuh",
                              "bart_internal.cuh")]
@@ -661,6 +663,8 @@ def run_native(args):
                          "note": (f"{FLOPS_PER_EVAL} algorithmic FP32 flops per line-point evaluation "
                                   f"(frac_16flop: the same time with {RATIONAL_FLOPS_PER_EVAL}); peak = "
                                   f"{n_sm} SMs x 128 FP32 lanes x 2 x {max_mhz:.0f} MHz (max SM clock); "
+                                  f"line-point evaluations are counted whether a line enters on its own or "
+                                  f"through its block's moments, so the fractions can exceed 1; "
                                   f"launch time = opacity-build events / {OPACITY_LAUNCHES_PER_STEP}")},
             "forward_model": fw,
             "parity": parity,
