@@ -21,7 +21,9 @@
 //      Gauss-Legendre angle from the running vertical optical depth, and the
 //      flux as a sum over layers of the layer-mean source times the drop of
 //      the quadrature-weighted transmittance (the angle sum taken inside the
-//      layer sum, so no per-angle state is kept);
+//      layer sum, so no per-angle state is kept); a thread takes one such
+//      pair or two (P), with two a warp's column ends where the rest of it
+//      cannot change its fluxes (OPAQUE_SHARE);
 //   3. writes the spectrum and the tile's band partial sums; the CTA that
 //      finishes a proposal's last tile sums its partials in a fixed order
 //      (FP64) into the band values.
@@ -110,6 +112,22 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned i
                : "memory");
 }
 
+// With two pairs a thread, a warp's column ends where twice the largest Planck
+// function of the profile times the transmittance left is below this share of
+// the flux gathered so far at every wavenumber: what lies below adds at most
+// that (the layers' terms telescope), a quarter of the flux's rounding.  The
+// rows below are not read, which is the point: 2,048 proposals on the 100-layer
+// grid read 655 GB from L2 if they read every layer (18 TB/s at 36.3 ms), and
+// 36% of the layers of prior draws lie below.
+constexpr float OPAQUE_SHARE = 1.0f / (float)(1 << 26);
+// Levels between two looks; two with the optical-depth limit, which ends
+// columns by the same test.  2,048 proposals: 36.3 ms with one pair and no
+// looks, 33.6 with two pairs, 28.0 with looks (29-30 with looks inside the level
+// loop).  One pair a thread (30.9 ms with looks) takes none: its looks cost 8%
+// of 301 ragged spectra on odd rows down to a cloud deck (642 us), where few
+// columns end early.
+constexpr int LOOK_EVERY = 8, LOOK_EVERY_TAU_LIM = 2;
+
 struct FusedArgs {
   const float* grid;                 // [S][L][M][N]
   int L, M;
@@ -154,6 +172,11 @@ struct FusedArgs {
 #ifndef FUSED_OCC_THREADS
 #define FUSED_OCC_THREADS 768
 #endif
+// The same for threads of two pairs (128 registers).
+#ifndef FUSED_OCC_THREADS2
+#define FUSED_OCC_THREADS2 512
+#endif
+constexpr int fused_occ_threads(int pairs) { return pairs == 1 ? FUSED_OCC_THREADS : FUSED_OCC_THREADS2; }
 
 // Two wavenumbers per thread, their arithmetic on packed FP32 pairs
 // (FFMA2/FADD2/FMUL2 of sm_100+: one issue slot for both); the MUFU
@@ -217,17 +240,23 @@ __device__ __forceinline__ float2 planck_pair(float2 c1nu3, float nu_a, float y,
   return mul2(mul2(c1nu3, f2(R)), em1);
 }
 
-// TW wavenumbers per tile, TW / 2 threads per CTA.
-template <int S, int NA, int TW, int MODE>
-__global__ void __launch_bounds__(TW / 2, FUSED_OCC_THREADS / (TW / 2))
+// NT threads per CTA with P pairs of neighbouring wavenumbers each: tiles of
+// 2 P NT wavenumbers.  Two pairs (P = 2) read a grid row by one 16-byte load
+// and share the layer record's reads and the row addresses, which takes rows
+// that start on 16-byte boundaries (n_nu a multiple of 4, 16-byte aligned
+// grid), and end columns early (OPAQUE_SHARE).  What bounds both is the row
+// reads: L2 output 69% busy, L1 hits 8%, load pipe 65%, issue 56% (two pairs,
+// 2,048 proposals on 4,096 wavenumbers).
+template <int S, int NA, int NT, int P, int MODE>
+__global__ void __launch_bounds__(NT, fused_occ_threads(P) / NT)
 emission_fused_kernel(const __grid_constant__ FusedArgs a) {
-  constexpr int NT = TW / 2;
+  constexpr int TW = 2 * P * NT;
   constexpr int NCF = LayerRec<S>::NCF;
   __shared__ LayerRec<S> s_rec[MAX_LAYERS];
   __shared__ float s_xs[S];
   __shared__ float2 s_red[NT / 32 > 0 ? NT / 32 : 1][MAX_BANDS];
   __shared__ unsigned long long s_unit;
-  __shared__ int s_last, s_ready;
+  __shared__ int s_last, s_ready, s_ymin;
   constexpr bool WIDE_X = (MODE & 1) != 0, TAU_LIM = (MODE & 2) != 0;
   const int tid = threadIdx.x;
   const int L = a.L, nb = a.n_bands;
@@ -267,7 +296,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         skip = true;
       }
     }
-    const int64_t lo2 = lo & ~(int64_t)1;          // tiles start on even indices (pairs)
+    const int64_t lo2 = lo & ~(int64_t)(2 * P - 1);   // tiles start on even indices (pairs), multiples of 4 (two pairs)
     const int n_tiles_p = skip ? 0 : (int)((hi - lo2 + TW - 1) / TW);
     const int n_groups_p = (n_tiles_p + a.tpu - 1) / a.tpu;
     if (!skip && grp < n_groups_p) {
@@ -275,7 +304,10 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
       // computed by the first unit of the proposal and published for the
       // others (a unit that finds them unpublished computes them itself),
       // and from them the layer records
-      if (tid == 0) s_ready = (ld_acquire(a.tw_flag + p) == ready_mark);
+      if (tid == 0) {
+        s_ready = (ld_acquire(a.tw_flag + p) == ready_mark);
+        s_ymin = 0x7f800000;                       // (read with two pairs alone)
+      }
       if (tid < S) {
         const float ab = a.theta ? a.theta[(int64_t)p * a.n_theta + 5 + tid] : 0.0f;
         s_xs[tid] = a.x0mu[tid] * exp10f(ab);
@@ -319,29 +351,33 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         }
         const float y = r.c2_t * LOG2E;
         s_rec[k].pl = make_float4(y, k > 0 ? __ldg(a.dpg + k - 1) : 0.0f, exp2f(y * dnu_f), 0.0f);
+        if (P == 2) atomicMin(&s_ymin, __float_as_int(y));   // of positive values: the hottest level
       }
       __syncthreads();
       if (!ready && tid == 0) st_release(a.tw_flag + p, ready_mark);   // publishes the CTA's stores above
       float2 band_acc = make_float2(0.f, 0.f);      // thread b < nb: band b over the unit's tiles
       const int t_end = min((grp + 1) * a.tpu, n_tiles_p);
 
-      // 2. the columns of wavenumbers ja and ja + 1 of one tile; PAIR: both
-      // read by one 8-byte load per row
+      // 2. the columns of wavenumbers ja .. ja + 2 P - 1 of one tile; PAIR:
+      // read by one load per row (always for P = 2)
       auto column = [&](auto pair_c, int tile) {
         constexpr bool PAIR = decltype(pair_c)::value;
-        const int64_t ja = lo2 + (int64_t)tile * TW + 2 * tid, jb = ja + 1;
-        const bool act_a = ja >= lo && ja < hi, act_b = jb < hi;
+        const int64_t ja = lo2 + (int64_t)tile * TW + 2 * P * tid;
         // idle lanes compute on valid indices
-        const int64_t ka = (ja < hi) ? ja : lo2, kb = (jb < hi) ? jb : ka;
+        const int64_t ka = (ja < hi) ? ja : lo2, kb = (P == 2 || ja + 1 < hi) ? ka + 1 : ka;
         // the wavenumbers from their FP64 positions, the rest in FP32
-        const float2 nuf = make_float2((float)(a.nu_start + (double)ka * a.dnu), (float)(a.nu_start + (double)kb * a.dnu));
-        constexpr float C1 = (float)(2.0 * bartc::H * bartc::C * bartc::C);
-        const float2 c1nu3 = mul2(mul2(f2(C1), nuf), mul2(nuf, nuf));
-        // Rayleigh a nu^4 / (mu m_u) (in FP64: a / (mu m_u) may be below the FP32 range)
-        float2 chi_r = f2(0.0f);
-        if (a.ex.ray != 0.0) {
-          const double nua = a.nu_start + (double)ka * a.dnu, nub = a.nu_start + (double)kb * a.dnu;
-          chi_r = make_float2((float)(a.ex.ray * (nua * nua) * (nua * nua)), (float)(a.ex.ray * (nub * nub) * (nub * nub)));
+        float2 nuf[P], c1nu3[P], chi_r[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+          const double nua = a.nu_start + (double)(ka + 2 * q) * a.dnu, nub = a.nu_start + (double)(kb + 2 * q) * a.dnu;
+          nuf[q] = make_float2((float)nua, (float)nub);
+          constexpr float C1 = (float)(2.0 * bartc::H * bartc::C * bartc::C);
+          c1nu3[q] = mul2(mul2(f2(C1), nuf[q]), mul2(nuf[q], nuf[q]));
+          // Rayleigh a nu^4 / (mu m_u) (in FP64: a / (mu m_u) may be below the FP32 range)
+          chi_r[q] = f2(0.0f);
+          if (a.ex.ray != 0.0)
+            chi_r[q] = make_float2((float)(a.ex.ray * (nua * nua) * (nua * nua)),
+                                   (float)(a.ex.ray * (nub * nub) * (nub * nub)));
         }
         const float* ga = a.grid + ka;
         const unsigned int dkb = (unsigned int)(kb - ka);
@@ -349,11 +385,11 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         // (tau the vertical optical depth from the top, ang_i = -log2(e)/mu_i)
         // only through their quadrature sum Tw = sum_i 2 pi w_i mu_i / 2 t_i,
         // so F = sum_k (B_{k-1} + B_k) (Tw_{k-1} - Tw_k) + 2 B_bottom Tw_bottom
-        float2 tau = f2(0.0f), Tw_prev = f2(a.tw_top), F = f2(0.0f);
+        float2 tau[P], Tw_prev[P], F[P], chi_prev[P], B_prev[P], B_hot[P];
         const int L_run = a.ex.L_run;
-        // grid values of a layer for both wavenumbers: lower (x) and upper (y)
-        // temperature bracket per species
-        auto fetch = [&](int k, float2* x, float2* y) {
+        // grid values of a layer: lower (x) and upper (y) temperature bracket
+        // per species
+        auto fetch = [&](int k, float2 (*x)[P], float2 (*y)[P]) {
           unsigned int of[4 * NCF];
 #pragma unroll
           for (int q = 0; q < NCF; ++q) {
@@ -365,16 +401,23 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           }
 #pragma unroll
           for (int q = 0; q < S; ++q) {
-            if (PAIR) {                            // ka is even and ka + 1 < N here
-              x[q] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q]));
-              y[q] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q + 1]));
+            if (P == 2) {                          // ka is a multiple of 4 and ka + 3 < N here
+              const float4 u = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q]));
+              const float4 v = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q + 1]));
+              x[q][0] = make_float2(u.x, u.y);
+              x[q][P - 1] = make_float2(u.z, u.w);
+              y[q][0] = make_float2(v.x, v.y);
+              y[q][P - 1] = make_float2(v.z, v.w);
+            } else if (PAIR) {                     // ka is even and ka + 1 < N here
+              x[q][0] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q]));
+              y[q][0] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q + 1]));
             } else {
-              x[q] = make_float2(__ldg(ga + of[2 * q]), __ldg(ga + (of[2 * q] + dkb)));
-              y[q] = make_float2(__ldg(ga + of[2 * q + 1]), __ldg(ga + (of[2 * q + 1] + dkb)));
+              x[q][0] = make_float2(__ldg(ga + of[2 * q]), __ldg(ga + (of[2 * q] + dkb)));
+              y[q][0] = make_float2(__ldg(ga + of[2 * q + 1]), __ldg(ga + (of[2 * q + 1] + dkb)));
             }
           }
         };
-        auto chi_of = [&](int k, const float2* x, const float2* y) {
+        auto chi_of = [&](int k, const float2 (*x)[P], const float2 (*y)[P], float2* chi) {
           float cf[4 * NCF];
 #pragma unroll
           for (int q = 0; q < NCF; ++q) {
@@ -384,88 +427,129 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
             cf[4 * q + 2] = v.z;
             cf[4 * q + 3] = v.w;
           }
-          float2 chi = chi_r;
 #pragma unroll
-          for (int q = 0; q < S; ++q) {
-            chi = fma2(f2(cf[2 * q]), x[q], chi);
-            chi = fma2(f2(cf[2 * q + 1]), y[q], chi);
+          for (int i = 0; i < P; ++i) {
+            chi[i] = chi_r[i];
+#pragma unroll
+            for (int q = 0; q < S; ++q) {
+              chi[i] = fma2(f2(cf[2 * q]), x[q][i], chi[i]);
+              chi[i] = fma2(f2(cf[2 * q + 1]), y[q][i], chi[i]);
+            }
           }
-          return chi;
         };
-        auto planck_k = [&](const float4& pl) {
-          if (WIDE_X) return planck2<true>(c1nu3, mul2(nuf, f2(pl.x)));
-          return planck_pair(c1nu3, nuf.x, pl.x, pl.z);
+        auto planck_k = [&](const float4& pl, float2* B) {
+#pragma unroll
+          for (int i = 0; i < P; ++i)
+            B[i] = WIDE_X ? planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(pl.x))) : planck_pair(c1nu3[i], nuf[i].x, pl.x, pl.z);
         };
-        float2 cx[S], cy[S], nx[S], ny[S];
+        float2 cx[S][P], cy[S][P], nx[S][P], ny[S][P];
         fetch(0, cx, cy);
         fetch(min(1, L_run - 1), nx, ny);
-        float2 chi_prev = chi_of(0, cx, cy);
-        float2 B_prev = planck_k(s_rec[0].pl);
-        bool done_a = false, done_b = false;       // lane reached the optical-depth limit
-#pragma unroll 2
-        for (int k = 1; k < L_run; ++k) {
+        chi_of(0, cx, cy, chi_prev);
+        planck_k(s_rec[0].pl, B_prev);
+        const float y_hot = __int_as_float(s_ymin);
 #pragma unroll
-          for (int q = 0; q < S; ++q) {
-            cx[q] = nx[q];
-            cy[q] = ny[q];
-          }
-          fetch(min(k + 1, L_run - 1), nx, ny);    // the next layer's rows are in flight meanwhile
-          const float2 chi = chi_of(k, cx, cy);
-          const float4 pl = s_rec[k].pl;
-          const float2 B = planck_k(pl);
-          const float2 dtau = mul2(add2(chi_prev, chi), f2(pl.y));
-          const float2 Bsum = add2(B_prev, B);
-          tau = add2(tau, dtau);
-          float2 Tw0 = f2(0.0f), Tw1 = f2(0.0f);    // two partial sums: a shorter dependence chain
-#pragma unroll
-          for (int i = 0; i < NA; ++i) {
-            const float2 t = ex2_2(mul2(tau, f2(a.ang[i])));
-            if (i & 1) Tw1 = fma2(f2(a.ang[NA + i]), t, Tw1);
-            else Tw0 = fma2(f2(a.ang[NA + i]), t, Tw0);
-          }
-          const float2 Tw = add2(Tw0, Tw1);
-          const float2 Fn = fma2(Bsum, sub2(Tw_prev, Tw), F);
-          chi_prev = chi;
-          if (!TAU_LIM) {
-            F = Fn;
-            Tw_prev = Tw;
-            B_prev = B;
-          } else {
-            // Sec. 4 item 7: stop at the caller's optical-depth limit; the level
-            // reached is the bottom boundary (its blackbody below).  Each
-            // wavenumber of the pair keeps its state from the level where it
-            // stopped while the other goes on.
-            if (!done_a) {
-              F.x = Fn.x;
-              Tw_prev.x = Tw.x;
-              B_prev.x = B.x;
-            }
-            if (!done_b) {
-              F.y = Fn.y;
-              Tw_prev.y = Tw.y;
-              B_prev.y = B.y;
-            }
-            done_a = done_a || tau.x > a.ex.tau_cut;
-            done_b = done_b || tau.y > a.ex.tau_cut;
-            if (done_a && done_b) break;
-          }
+        for (int i = 0; i < P; ++i) {
+          tau[i] = F[i] = f2(0.0f);
+          Tw_prev[i] = f2(a.tw_top);
+          // no level's Planck function is larger (up to rounding) than the hottest one's
+          B_hot[i] = mul2(f2(2.0f / OPAQUE_SHARE), planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(y_hot))));
         }
-        F = fma2(mul2(f2(2.0f), B_prev), Tw_prev, F);   // the bottom level's blackbody through the column
-        if (a.spectra) {
-          const int64_t base = (a.offs ? a.offs[p] : (int64_t)p * a.N) - lo;
-          if (act_a) a.spectra[base + ja] = F.x;
-          if (act_b) a.spectra[base + jb] = F.y;
+        bool done_a[P] = {}, done_b[P] = {};       // lane reached the optical-depth limit
+        for (int k = 1; k < L_run;) {
+          const int k_look = P == 1 ? L_run : min(k + (TAU_LIM ? LOOK_EVERY_TAU_LIM : LOOK_EVERY), L_run);
+#pragma unroll 2
+          for (; k < k_look; ++k) {
+            float2 chi[P], B[P];
+            if (P == 1) {
+#pragma unroll
+              for (int q = 0; q < S; ++q) {
+                cx[q][0] = nx[q][0];
+                cy[q][0] = ny[q][0];
+              }
+              fetch(min(k + 1, L_run - 1), nx, ny);  // the next layer's rows are in flight meanwhile
+              chi_of(k, cx, cy, chi);
+            } else {                                 // one set of rows in registers
+              chi_of(k, nx, ny, chi);
+              fetch(min(k + 1, L_run - 1), nx, ny);
+            }
+            const float4 pl = s_rec[k].pl;
+            planck_k(pl, B);
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+              tau[i] = add2(tau[i], mul2(add2(chi_prev[i], chi[i]), f2(pl.y)));
+              chi_prev[i] = chi[i];
+              const float2 Bsum = add2(B_prev[i], B[i]);
+              float2 Tw0 = f2(0.0f), Tw1 = f2(0.0f);   // two partial sums: a shorter dependence chain
+#pragma unroll
+              for (int q = 0; q < NA; ++q) {
+                const float2 t = ex2_2(mul2(tau[i], f2(a.ang[q])));
+                if (q & 1) Tw1 = fma2(f2(a.ang[NA + q]), t, Tw1);
+                else Tw0 = fma2(f2(a.ang[NA + q]), t, Tw0);
+              }
+              const float2 Tw = add2(Tw0, Tw1);
+              const float2 Fn = fma2(Bsum, sub2(Tw_prev[i], Tw), F[i]);
+              if (!TAU_LIM) {
+                F[i] = Fn;
+                Tw_prev[i] = Tw;
+                B_prev[i] = B[i];
+              } else {
+                // Sec. 4 item 7: stop at the caller's optical-depth limit; the level
+                // reached is the bottom boundary (its blackbody below).  Each
+                // wavenumber keeps its state from the level where it stopped
+                // while the others go on.
+                if (!done_a[i]) {
+                  F[i].x = Fn.x;
+                  Tw_prev[i].x = Tw.x;
+                  B_prev[i].x = B[i].x;
+                }
+                if (!done_b[i]) {
+                  F[i].y = Fn.y;
+                  Tw_prev[i].y = Tw.y;
+                  B_prev[i].y = B[i].y;
+                }
+                done_a[i] = done_a[i] || tau[i].x > a.ex.tau_cut;
+                done_b[i] = done_b[i] || tau[i].y > a.ex.tau_cut;
+              }
+            }
+            if (P == 1 && TAU_LIM && done_a[0] && done_b[0]) break;
+          }
+          if (P == 1) break;
+          bool over = true;                          // (all lanes of a warp take the same levels)
+#pragma unroll
+          for (int i = 0; i < P; ++i) {
+            const float2 rest = mul2(B_hot[i], Tw_prev[i]);
+            over = over && (done_a[i] || rest.x <= F[i].x) && (done_b[i] || rest.y <= F[i].y);
+          }
+          if (__all_sync(0xffffffffu, over)) break;
+        }
+        const int64_t base = a.spectra ? (a.offs ? a.offs[p] : (int64_t)p * a.N) - lo : 0;
+        float dw[2 * P], Fw[2 * P];                // trapezoid weights (0: not this span's), fluxes
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+          F[i] = fma2(mul2(f2(2.0f), B_prev[i]), Tw_prev[i], F[i]);   // the bottom level's blackbody through the column
+          Fw[2 * i] = F[i].x;
+          Fw[2 * i + 1] = F[i].y;
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * P; ++i) {
+          const int64_t j = ja + i;
+          const bool act = j >= lo && j < hi;
+          dw[i] = act ? ((hi - lo == 1) ? 1.0f : ((j == lo || j == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
+          if (a.spectra && act) a.spectra[base + j] = Fw[i];
         }
 
         // 3. band sums of the tile, added to the unit's
         if (nb > 0) {
-          const float dwa = act_a ? ((hi - lo == 1) ? 1.0f : ((ja == lo || ja == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
-          const float dwb = act_b ? ((hi - lo == 1) ? 1.0f : ((jb == lo || jb == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
           const int warp = tid >> 5, lane = tid & 31;
           for (int b = 0; b < nb; ++b) {
-            const float Wa = act_a ? __ldg(a.filt + (int64_t)b * a.N + ja) * dwa : 0.0f;
-            const float Wb = act_b ? __ldg(a.filt + (int64_t)b * a.N + jb) * dwb : 0.0f;
-            float num = fmaf(Wa, F.x, Wb * F.y), den = Wa + Wb;
+            float num = 0.0f, den = 0.0f;
+#pragma unroll
+            for (int i = 2 * P - 1; i >= 0; --i) {
+              const float Wi = dw[i] > 0.0f ? __ldg(a.filt + (int64_t)b * a.N + ja + i) * dw[i] : 0.0f;
+              num = fmaf(Wi, Fw[i], num);
+              den += Wi;
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
               num += __shfl_xor_sync(0xffffffffu, num, o);
@@ -485,8 +569,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         }
       };
       for (int tile = grp * a.tpu; tile < t_end; ++tile) {
-        if (pair_loads) column(std::true_type{}, tile);
-        else column(std::false_type{}, tile);
+        if (P == 2 || pair_loads) column(std::true_type{}, tile);
+        else if (P == 1) column(std::integral_constant<bool, P == 2>{}, tile);   // (only P = 1 has the form)
       }
 
       // the unit's band partials; the proposal's last unit reduces them
@@ -859,19 +943,19 @@ emission_tma_kernel(const __grid_constant__ FusedArgs a) {
 
 using FusedLauncher = cudaError_t (*)(const FusedArgs&, int, cudaStream_t);
 
-// Wavenumbers per tile the autotuner chooses from (two per compute thread;
-// at least 128, so a CTA has a thread for each of up to 64 bands).
-constexpr int FUSED_TILES[3] = {128, 256, 512};
+// Threads per CTA the autotuner chooses from (at least 64, so a CTA has one
+// for each of up to 64 bands), 2 wavenumbers each or 4.
+constexpr int FUSED_THREADS[3] = {64, 128, 256};
 
-template <int S, int NA, int TW, int MODE>
+template <int S, int NA, int NT, int P, int MODE>
 cudaError_t launch_pair(const FusedArgs& a, int sm_count, cudaStream_t st) {
   int per_sm = 0;
   cudaError_t e =
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, emission_fused_kernel<S, NA, TW, MODE>, TW / 2, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, emission_fused_kernel<S, NA, NT, P, MODE>, NT, 0);
   if (e != cudaSuccess) return e;
   unsigned long long grid = (unsigned long long)(per_sm < 1 ? 1 : per_sm) * (unsigned long long)sm_count;
   if (grid > a.n_units) grid = a.n_units;
-  emission_fused_kernel<S, NA, TW, MODE><<<(unsigned)grid, TW / 2, 0, st>>>(a);
+  emission_fused_kernel<S, NA, NT, P, MODE><<<(unsigned)grid, NT, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -890,48 +974,61 @@ cudaError_t launch_tma(const FusedArgs& a, int sm_count, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Launcher of the fused generation for S species and na angles at tile tw:
-// the bulk-copy kernel (tma; its options are run-time flags), else the
-// global-load kernel with the compile-time mode (bit 0 FP64 Planck branch,
-// bit 1 optical-depth limit).  Instantiated once per species count, each in
-// its own translation unit.
+// Forms of the fused launch: pairs of wavenumbers per thread, or bulk copies
+// (pairs).
+enum FusedForm { FUSED_PAIR, FUSED_TWO_PAIRS, FUSED_BULK };
+constexpr int fused_width(FusedForm f, int nt) { return (f == FUSED_TWO_PAIRS ? 4 : 2) * nt; }   // tile
+
+// Launcher of the fused generation for S species and na angles with nt
+// (compute) threads per CTA: the bulk-copy kernel (its options are run-time
+// flags), else the global-load kernel with the compile-time mode (bit 0 FP64
+// Planck branch, bit 1 optical-depth limit).  Instantiated once per species
+// count, each in its own translation unit.
 template <int S>
-FusedLauncher fused_launcher(int na, bool tma, int tw, int mode);
+FusedLauncher fused_launcher(int na, FusedForm form, int nt, int mode);
 
-extern template FusedLauncher fused_launcher<1>(int, bool, int, int);
-extern template FusedLauncher fused_launcher<2>(int, bool, int, int);
-extern template FusedLauncher fused_launcher<3>(int, bool, int, int);
-extern template FusedLauncher fused_launcher<4>(int, bool, int, int);
+extern template FusedLauncher fused_launcher<1>(int, FusedForm, int, int);
+extern template FusedLauncher fused_launcher<2>(int, FusedForm, int, int);
+extern template FusedLauncher fused_launcher<3>(int, FusedForm, int, int);
+extern template FusedLauncher fused_launcher<4>(int, FusedForm, int, int);
 
-template <int S, int NA, int TW>
-FusedLauncher pick_mode(bool tma, int mode) {
-  if (tma) return launch_tma<S, NA, TW>;
+template <int S, int NA, int NT, int P>
+FusedLauncher pick_mode(int mode) {
   switch (mode) {
-    case 0: return launch_pair<S, NA, TW, 0>;
-    case 1: return launch_pair<S, NA, TW, 1>;
-    case 2: return launch_pair<S, NA, TW, 2>;
-    default: return launch_pair<S, NA, TW, 3>;
+    case 0: return launch_pair<S, NA, NT, P, 0>;
+    case 1: return launch_pair<S, NA, NT, P, 1>;
+    case 2: return launch_pair<S, NA, NT, P, 2>;
+    default: return launch_pair<S, NA, NT, P, 3>;
+  }
+}
+
+template <int S, int NA, int NT>
+FusedLauncher pick_form(FusedForm form, int mode) {
+  switch (form) {
+    case FUSED_BULK: return launch_tma<S, NA, 2 * NT>;
+    case FUSED_TWO_PAIRS: return pick_mode<S, NA, NT, 2>(mode);
+    default: return pick_mode<S, NA, NT, 1>(mode);
   }
 }
 
 template <int S, int NA>
-FusedLauncher pick_tile(bool tma, int tw, int mode) {
-  switch (tw) {
-    case 128: return pick_mode<S, NA, 128>(tma, mode);
-    case 256: return pick_mode<S, NA, 256>(tma, mode);
-    case 512: return pick_mode<S, NA, 512>(tma, mode);
+FusedLauncher pick_tile(FusedForm form, int nt, int mode) {
+  switch (nt) {
+    case 64: return pick_form<S, NA, 64>(form, mode);
+    case 128: return pick_form<S, NA, 128>(form, mode);
+    case 256: return pick_form<S, NA, 256>(form, mode);
     default: return nullptr;
   }
 }
 
 template <int S>
-FusedLauncher fused_launcher(int na, bool tma, int tw, int mode) {
+FusedLauncher fused_launcher(int na, FusedForm form, int nt, int mode) {
   switch (na) {
-    case 1: return pick_tile<S, 1>(tma, tw, mode);
-    case 2: return pick_tile<S, 2>(tma, tw, mode);
-    case 4: return pick_tile<S, 4>(tma, tw, mode);
-    case 8: return pick_tile<S, 8>(tma, tw, mode);
-    case 16: return pick_tile<S, 16>(tma, tw, mode);
+    case 1: return pick_tile<S, 1>(form, nt, mode);
+    case 2: return pick_tile<S, 2>(form, nt, mode);
+    case 4: return pick_tile<S, 4>(form, nt, mode);
+    case 8: return pick_tile<S, 8>(form, nt, mode);
+    case 16: return pick_tile<S, 16>(form, nt, mode);
     default: return nullptr;
   }
 }

@@ -14,12 +14,12 @@ using namespace bartem;
 
 namespace {
 
-FusedLauncher pick_fused(int S, int na, bool tma, int tw, int mode) {
+FusedLauncher pick_fused(int S, int na, FusedForm form, int nt, int mode) {
   switch (S) {
-    case 1: return fused_launcher<1>(na, tma, tw, mode);
-    case 2: return fused_launcher<2>(na, tma, tw, mode);
-    case 3: return fused_launcher<3>(na, tma, tw, mode);
-    case 4: return fused_launcher<4>(na, tma, tw, mode);
+    case 1: return fused_launcher<1>(na, form, nt, mode);
+    case 2: return fused_launcher<2>(na, form, nt, mode);
+    case 3: return fused_launcher<3>(na, form, nt, mode);
+    case 4: return fused_launcher<4>(na, form, nt, mode);
     default: return nullptr;
   }
 }
@@ -33,9 +33,16 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   const int mode = emission_mode(g, c);
   // the bulk-copy variant on request, where its 16-byte row starts hold:
   // n_nu a multiple of 4 and an aligned grid
-  const bool tma = ctx->em_launch == BART_LAUNCH_FUSED_TMA && (N % 4 == 0) &&
-                   (reinterpret_cast<uintptr_t>(g->grid) % 16 == 0);
-  if (S > FUSED_MAX_SPECIES || !pick_fused(S, NA, tma, FUSED_TILES[1], mode))
+  const bool rows16 = (N % 4 == 0) && (reinterpret_cast<uintptr_t>(g->grid) % 16 == 0);
+  // else two pairs per thread where the rows allow it and the call has enough
+  // wavenumbers to fill the SMs twice with such threads (16 proposals on 100,000
+  // wavenumbers: 418 us in pairs, 370 with two; 354 on 1,600, a fill and a half:
+  // 80 us in pairs, 84 with two)
+  const FusedForm form = !rows16 ? FUSED_PAIR
+                         : ctx->em_launch == BART_LAUNCH_FUSED_TMA ? FUSED_BULK
+                         : (double)n * (double)N >= 8.0 * FUSED_OCC_THREADS2 * ctx->sm_count ? FUSED_TWO_PAIRS
+                                                                                            : FUSED_PAIR;
+  if (S > FUSED_MAX_SPECIES || !pick_fused(S, NA, form, FUSED_THREADS[1], mode))
     return bart_fail(ctx, BART_EUNSUPPORTED, "emission with %d species and %d angles is not instantiated "
                      "(species 1-4; angles 1, 2, 4, 8, 16)", S, NA);
   bart_status st;
@@ -52,7 +59,7 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   if ((st = bart_scratch(ctx, "ff_work", 3 * sizeof(unsigned long long), &p_work)) != BART_OK) return st;
   if ((st = bart_scratch(ctx, "ff_twc", (size_t)n * L * sizeof(LayerTW), &p_twc)) != BART_OK) return st;
   if ((st = bart_scratch(ctx, "ff_flag", (size_t)n * sizeof(unsigned int), &p_flag)) != BART_OK) return st;
-  const int max_tiles = (int)((N + 3 + FUSED_TILES[0] - 1) / FUSED_TILES[0]);   // smallest tile, aligned start
+  const int max_tiles = (int)((N + 3 + 2 * FUSED_THREADS[0] - 1) / (2 * FUSED_THREADS[0]));   // smallest tile, aligned start
   if (nb > 0) {
     if ((st = bart_scratch(ctx, "ff_done", (size_t)n * sizeof(unsigned int), &p_done)) != BART_OK) return st;
     if ((st = bart_scratch(ctx, "fw_part", (size_t)n * max_tiles * nb * sizeof(float2), &p_part)) != BART_OK)
@@ -118,34 +125,34 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   }
   const long long span_cap =
       (l2_bytes > 0 ? (long long)l2_bytes / 2 : (64LL << 20)) / ((long long)S * L * M * (long long)sizeof(float));
-  auto run = [&](int tw) -> bart_status {
+  auto run = [&](int nt) -> bart_status {
+    const int tw = fused_width(form, nt);
     // several consecutive tiles per unit amortise the unit's fixed work (layer
     // states, band partials and counts), as long as there are enough units to
     // balance the CTAs (about 8 per CTA of a full grid)
     const int n_tiles = (int)((N + 3 + tw - 1) / tw);                // tiles start on an aligned index
-    const long long target = 8LL * ctx->sm_count * (2 * FUSED_OCC_THREADS / tw);
+    const long long target = 8LL * ctx->sm_count * (fused_occ_threads(form == FUSED_TWO_PAIRS ? 2 : 1) / nt);
     const long long tpu_cap = std::max(1LL, std::min<long long>(MAX_TILES_PER_UNIT, span_cap / tw));
     a.tpu = (int)std::max(1LL, std::min<long long>(tpu_cap, (long long)n * n_tiles / target));
     a.n_groups = (n_tiles + a.tpu - 1) / a.tpu;
     a.n_units = (unsigned long long)a.n_groups * (unsigned long long)n;
-    cudaError_t e = pick_fused(S, NA, tma, tw, mode)(a, ctx->sm_count, ctx->stream);
+    cudaError_t e = pick_fused(S, NA, form, nt, mode)(a, ctx->sm_count, ctx->stream);
     if (e != cudaSuccess) return bart_fail(ctx, BART_ECUDA, "launch of emission_fused_kernel failed: %s",
                                            cudaGetErrorString(e));
     return BART_OK;
   };
-  // tile width: fixed by the caller, cached per shape, or measured once
+  // threads per CTA: fixed by the caller, cached per shape, or measured once
   // (each candidate timed with CUDA events on the stream) outside a capture
   char key[160];
-  snprintf(key, sizeof(key), "fused%s S%d A%d L%d/%d M%d N%lld n%d b%d span%d m%d", tma ? " tma" : "", S, NA, L,
+  snprintf(key, sizeof(key), "fused%s S%d A%d L%d/%d M%d N%lld n%d b%d span%d m%d", form == FUSED_BULK ? " tma" : form == FUSED_TWO_PAIRS ? " x4" : "", S, NA, L,
            a.ex.L_run, M, (long long)N, n, nb, b->nu_lo ? 1 : 0, mode);
-  // the caller's width is in threads of the one-wavenumber-per-thread
-  // kernels; here a compute thread takes two
-  int tw = ctx->em_tile > 0 ? 2 * ctx->em_tile : FUSED_TILES[1];
+  // (the caller's width is that of the one-wavenumber-per-thread kernels)
+  int nt = ctx->em_tile > 0 ? ctx->em_tile : FUSED_THREADS[1];
   auto it = ctx->tiles.find(key);
   if (ctx->em_tile > 0) {
     // fixed by the caller
   } else if (it != ctx->tiles.end()) {
-    tw = it->second;
+    nt = it->second / fused_width(form, 1);
   } else if (ctx->autotune) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     BART_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cs));
@@ -154,7 +161,7 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
       BART_CUDA(ctx, cudaEventCreate(&e0));
       BART_CUDA(ctx, cudaEventCreate(&e1));
       float best = 1e30f;
-      for (int cand : FUSED_TILES) {
+      for (int cand : FUSED_THREADS) {
         BART_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
         if ((st = run(cand)) != BART_OK) return st;
         BART_CUDA(ctx, cudaEventRecord(e1, ctx->stream));
@@ -163,13 +170,13 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
         BART_CUDA(ctx, cudaEventElapsedTime(&ms, e0, e1));
         if (ms < best) {
           best = ms;
-          tw = cand;
+          nt = cand;
         }
       }
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      ctx->tiles[key] = tw;
+      ctx->tiles[key] = fused_width(form, nt);
     }
   }
-  return run(tw);
+  return run(nt);
 }

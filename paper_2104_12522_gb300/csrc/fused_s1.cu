@@ -2,5 +2,5 @@
 #include "emission_fused.cuh"
 
 namespace bartem {
-template FusedLauncher fused_launcher<1>(int, bool, int, int);
+template FusedLauncher fused_launcher<1>(int, FusedForm, int, int);
 }  // namespace bartem

@@ -2,5 +2,5 @@
 #include "emission_fused.cuh"
 
 namespace bartem {
-template FusedLauncher fused_launcher<2>(int, bool, int, int);
+template FusedLauncher fused_launcher<2>(int, FusedForm, int, int);
 }  // namespace bartem
