@@ -122,7 +122,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned i
 constexpr float OPAQUE_SHARE = 1.0f / (float)(1 << 26);
 // Levels between two looks; two with the optical-depth limit, which ends
 // columns by the same test.  2,048 proposals: 36.3 ms with one pair and no
-// looks, 33.6 with two pairs, 28.0 with looks (29-30 with looks inside the level
+// looks, 33.6 with two pairs, 28.0-28.6 with looks (29-30 with looks inside the level
 // loop).  One pair a thread (30.9 ms with looks) takes none: its looks cost 8%
 // of 301 ragged spectra on odd rows down to a cloud deck (642 us), where few
 // columns end early.
@@ -245,7 +245,7 @@ __device__ __forceinline__ float2 planck_pair(float2 c1nu3, float nu_a, float y,
 // and share the layer record's reads and the row addresses, which takes rows
 // that start on 16-byte boundaries (n_nu a multiple of 4, 16-byte aligned
 // grid), and end columns early (OPAQUE_SHARE).  What bounds both is the row
-// reads: L2 output 69% busy, L1 hits 8%, load pipe 65%, issue 56% (two pairs,
+// reads: L2 output 74% busy, L1 hits 7%, load pipe 66%, issue 53% (two pairs,
 // 2,048 proposals on 4,096 wavenumbers).
 template <int S, int NA, int NT, int P, int MODE>
 __global__ void __launch_bounds__(NT, fused_occ_threads(P) / NT)
