@@ -89,6 +89,31 @@ void bart_scratch_give_back(bart_ctx* ctx, std::vector<void*>* held) {
   held->clear();
 }
 
+bart_status bart_call_memory(bart_ctx* ctx, size_t bytes, void** out) {
+  cudaError_t e = cudaSuccess;
+  if (stream_capturing(ctx)) {
+    e = cudaMallocAsync(out, bytes, ctx->stream);      // an allocation node of the graph
+  } else {
+    if (!ctx->pool) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = ctx->device;
+      unsigned long long kept = BART_POOL_KEPT;
+      e = cudaMemPoolCreate(&ctx->pool, &props);
+      if (e == cudaSuccess) e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &kept);
+    }
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(out, bytes, ctx->pool, ctx->stream);
+  }
+  if (e == cudaSuccess) return BART_OK;
+  cudaGetLastError();
+  return bart_fail(ctx, BART_ENOMEM, "%zu bytes of memory for this call: %s", bytes, cudaGetErrorString(e));
+}
+
+void bart_call_free(bart_ctx* ctx, void* p) {
+  if (p && cudaFreeAsync(p, ctx->stream) != cudaSuccess) cudaGetLastError();
+}
+
 bart_status bart_upload_const(bart_ctx* ctx, const char* name, const void* data, size_t bytes, void** dev) {
   void* before = nullptr;
   auto it0 = ctx->scratch.find(name);
@@ -136,6 +161,7 @@ extern "C" void bart_destroy(bart_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
   for (auto& kv : ctx->scratch) cudaFree(kv.second.first);
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->d_wtable) cudaFree(ctx->d_wtable);
   delete ctx;

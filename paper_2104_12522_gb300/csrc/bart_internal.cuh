@@ -32,6 +32,7 @@ struct bart_ctx {
   cudaStream_t user_stream = nullptr;  // the caller's stream while a capture is open
   bool capturing = false;           // between bart_capture_begin and bart_capture_end
   int* d_status = nullptr;          // device status word
+  cudaMemPool_t pool = nullptr;     // memory of single calls (bart_call_memory)
   float2* d_wtable = nullptr;       // Faddeeva Taylor-coefficient table
   bool wtable_ready = false;
 };
@@ -63,6 +64,15 @@ bart_status bart_scratch(bart_ctx* ctx, const char* name, size_t bytes, void** o
 // bart_scratch_give_back frees them after the last launch that uses them.
 bart_status bart_scratch_any(bart_ctx* ctx, const char* name, size_t bytes, void** out, std::vector<void*>* held);
 void bart_scratch_give_back(bart_ctx* ctx, std::vector<void*>* held);
+
+// Memory of one call, ordered on the context's stream: no other call, graph or
+// stream of the context ever shares it.  It comes from a pool of the context
+// that keeps at most BART_POOL_KEPT bytes between synchronisations; inside a
+// stream capture the graph itself allocates and frees it.  bart_call_free
+// follows the last launch that uses it.
+constexpr unsigned long long BART_POOL_KEPT = 64ULL << 20;
+bart_status bart_call_memory(bart_ctx* ctx, size_t bytes, void** out);
+void bart_call_free(bart_ctx* ctx, void* p);
 
 // Device copy of a small host constant buffer, kept in scratch `name`.  The
 // copy is issued only when the bytes differ from the last upload, so a call

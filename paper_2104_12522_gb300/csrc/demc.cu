@@ -816,22 +816,29 @@ extern "C" bart_status bart_chain_stats(bart_ctx* ctx, const float* chain, int n
   const int64_t series = (int64_t)n_chains * n_params;
   const int rows = std::max(64, (int)(((int64_t)n + ST_MAX_CHUNKS - 1) / ST_MAX_CHUNKS));
   const int n_chunks = (int)(((int64_t)n + rows - 1) / rows);
-  // Series are taken in batches whose scratch (12 n bytes a series for the lag
+  // Series are taken in batches whose memory (12 n bytes a series for the lag
   // sums: the centred series and the autocorrelations) stays within 512 MB,
-  // at least one series at a time.
+  // at least one series at a time, and in smaller ones where that is not free.
+  // It belongs to this call alone: calls on other streams of the context and
+  // graphs that captured one are independent of it.
   const int64_t per = (int64_t)n * 8 + (int64_t)(n / 2) * 8;
-  const int batch = (int)std::min<int64_t>(series, std::max<int64_t>(1, speis ? (512LL << 20) / per : 1 << 20));
+  int batch = (int)std::min<int64_t>(series, std::max<int64_t>(1, speis ? (512LL << 20) / per : 1 << 20));
   bart_status st;
   double *sums = nullptr, *sq = nullptr, *e = nullptr, *rho = nullptr, *tot = nullptr;
   int* first = nullptr;
-  std::vector<void*> held;
-  auto take = [&](const char* name, size_t bytes, void** out) { return bart_scratch_any(ctx, name, bytes, out, &held); };
-  st = take("st_sums", (size_t)n_chunks * batch * 8, (void**)&sums);
-  if (st == BART_OK) st = take("st_sq", (size_t)n_chunks * batch * 8, (void**)&sq);
-  if (st == BART_OK && speis) st = take("st_e", (size_t)batch * n * 8, (void**)&e);
-  if (st == BART_OK && speis) st = take("st_rho", (size_t)batch * (n / 2) * 8, (void**)&rho);
-  if (st == BART_OK && speis) st = take("st_first", (size_t)batch * 4, (void**)&first);
-  if (st == BART_OK && gr) st = take("st_tot", (size_t)series * 16, (void**)&tot);
+  for (;; batch = (batch + 1) / 2) {
+    const size_t part = (size_t)n_chunks * batch, rows_of = speis ? batch : 0;
+    const size_t doubles = 2 * part + rows_of * ((size_t)n + n / 2) + (gr ? 2 * (size_t)series : 0);
+    st = bart_call_memory(ctx, doubles * 8 + rows_of * 4, (void**)&sums);
+    if (st != BART_OK && batch > 1) continue;
+    if (st != BART_OK) return st;
+    sq = sums + part;
+    e = speis ? sq + part : nullptr;
+    rho = sq + part + rows_of * n;
+    tot = rho + rows_of * (n / 2);
+    first = reinterpret_cast<int*>(sums + doubles);
+    break;
+  }
   for (int64_t s0 = 0; st == BART_OK && s0 < series; s0 += batch) {
     const int m = (int)std::min<int64_t>(batch, series - s0);
     const dim3 grid((unsigned)((m + ST_SERIES - 1) / ST_SERIES), (unsigned)n_chunks);
@@ -855,6 +862,6 @@ extern "C" bart_status bart_chain_stats(bart_ctx* ctx, const float* chain, int n
     gr_kernel<<<n_params, ST_THREADS, 0, ctx->stream>>>(tot, tot + series, n, n_chains, n_params, gr);
     st = bart_check_launch(ctx, "gr_kernel");
   }
-  bart_scratch_give_back(ctx, &held);
+  bart_call_free(ctx, sums);
   return st;
 }
