@@ -125,7 +125,9 @@ bart_status bart_set_emission_launch(bart_ctx* ctx, int mode);
  * (otherwise they return BART_EINVAL and bart_capture_end fails).  A graph
  * keeps the device pointers it was captured with: replaying it recomputes
  * from whatever those buffers hold then (CUDA Graphs; the paper's sampler
- * calls the same forward model once per generation, Sec. 3). */
+ * calls the same forward model once per generation, Sec. 3).  Scratch that a
+ * graph was captured with keeps its address when later calls need more, until
+ * the context is destroyed. */
 typedef struct bart_graph bart_graph;
 bart_status bart_capture_begin(bart_ctx* ctx);
 bart_status bart_capture_end(bart_ctx* ctx, bart_graph** out);

@@ -29,6 +29,7 @@ bart_status bart_check_launch(bart_ctx* ctx, const char* what) {
 
 // True while work issued on the context's stream is being captured.
 static bool stream_capturing(bart_ctx* ctx) {
+  if (!ctx->stream || ctx->stream == cudaStreamLegacy) return false;   // cannot be captured
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess) {
     cudaGetLastError();
@@ -39,17 +40,23 @@ static bool stream_capturing(bart_ctx* ctx) {
 
 bart_status bart_scratch(bart_ctx* ctx, const char* name, size_t bytes, void** out) {
   auto it = ctx->scratch.find(name);
+  const bool captured = stream_capturing(ctx);
   if (it != ctx->scratch.end() && it->second.second >= bytes) {
+    if (captured && !ctx->own_capture) ctx->in_graph.insert(name);
     *out = it->second.first;
     return BART_OK;
   }
-  if (stream_capturing(ctx))
+  if (captured)
     return bart_fail(ctx, BART_EINVAL, "scratch '%s' (%zu bytes) must be sized by an eager call of the same "
                      "shape before a stream capture", name, bytes);
   if (it != ctx->scratch.end()) {
-    // The old buffer may still be in use by queued work on this stream.
-    BART_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    cudaFree(it->second.first);
+    if (ctx->in_graph.erase(name)) {
+      ctx->outgrown.push_back(it->second.first);
+    } else {
+      // The old buffer may still be in use by queued work on this stream.
+      BART_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+      cudaFree(it->second.first);
+    }
     ctx->scratch.erase(it);
   }
   void* p = nullptr;
@@ -161,6 +168,7 @@ extern "C" void bart_destroy(bart_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
   for (auto& kv : ctx->scratch) cudaFree(kv.second.first);
+  for (void* p : ctx->outgrown) cudaFree(p);
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->d_wtable) cudaFree(ctx->d_wtable);

@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 #include <map>
+#include <set>
 
 #include "../../include/bartgpu.h"
 
@@ -23,6 +24,10 @@ struct bart_ctx {
   std::string err;
   // Growable scratch: one buffer per purpose so calls can keep it resident.
   std::map<std::string, std::pair<void*, size_t>> scratch;
+  // Buffers that a caller's graph was captured with stay at their address when
+  // a later call outgrows them, until the context is destroyed.
+  std::set<std::string> in_graph;   // names of the scratch taken inside a capture
+  std::vector<void*> outgrown;
   std::map<std::string, std::vector<unsigned char>> uploaded;   // host copy of each constant buffer
   std::map<std::string, int> tiles;  // autotuned tile width per launch shape
   int autotune = 1;
@@ -30,6 +35,7 @@ struct bart_ctx {
   int em_tile = 0;                  // emission tile width fixed by the caller (0: autotuner)
   int em_launch = BART_LAUNCH_FUSED; // emission launch structure (bart_set_emission_launch)
   cudaStream_t user_stream = nullptr;  // the caller's stream while a capture is open
+  bool own_capture = false;         // the capture of bart_retrieval_run, whose graph ends with the call
   bool capturing = false;           // between bart_capture_begin and bart_capture_end
   int* d_status = nullptr;          // device status word
   cudaMemPool_t pool = nullptr;     // memory of single calls (bart_call_memory)

@@ -115,7 +115,9 @@ extern "C" bart_status bart_retrieval_run(bart_ctx* ctx, bart_demc* s, bart_mlp*
       bart_status rc = BART_OK;
       if (ce == cudaSuccess) {
         ctx->stream = cap;
+        ctx->own_capture = true;
         rc = generation();
+        ctx->own_capture = false;
         ctx->stream = st;
         ce = cudaStreamEndCapture(cap, &graph);   // always ends the capture
       }
