@@ -304,10 +304,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
       // computed by the first unit of the proposal and published for the
       // others (a unit that finds them unpublished computes them itself),
       // and from them the layer records
-      if (tid == 0) {
-        s_ready = (ld_acquire(a.tw_flag + p) == ready_mark);
-        s_ymin = 0x7f800000;                       // (read with two pairs alone)
-      }
+      if (tid == 0) s_ready = (ld_acquire(a.tw_flag + p) == ready_mark);
+      if (P == 2 && tid == 0) s_ymin = 0x7f800000;
       if (tid < S) {
         const float ab = a.theta ? a.theta[(int64_t)p * a.n_theta + 5 + tid] : 0.0f;
         s_xs[tid] = a.x0mu[tid] * exp10f(ab);
@@ -358,26 +356,23 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
       float2 band_acc = make_float2(0.f, 0.f);      // thread b < nb: band b over the unit's tiles
       const int t_end = min((grp + 1) * a.tpu, n_tiles_p);
 
-      // 2. the columns of wavenumbers ja .. ja + 2 P - 1 of one tile; PAIR:
-      // read by one load per row (always for P = 2)
+      // 2. one pair a thread: the columns of wavenumbers ja and ja + 1 of one
+      // tile; PAIR: both read by one 8-byte load per row
       auto column = [&](auto pair_c, int tile) {
         constexpr bool PAIR = decltype(pair_c)::value;
-        const int64_t ja = lo2 + (int64_t)tile * TW + 2 * P * tid;
+        const int64_t ja = lo2 + (int64_t)tile * TW + 2 * tid, jb = ja + 1;
+        const bool act_a = ja >= lo && ja < hi, act_b = jb < hi;
         // idle lanes compute on valid indices
-        const int64_t ka = (ja < hi) ? ja : lo2, kb = (P == 2 || ja + 1 < hi) ? ka + 1 : ka;
+        const int64_t ka = (ja < hi) ? ja : lo2, kb = (jb < hi) ? jb : ka;
         // the wavenumbers from their FP64 positions, the rest in FP32
-        float2 nuf[P], c1nu3[P], chi_r[P];
-#pragma unroll
-        for (int q = 0; q < P; ++q) {
-          const double nua = a.nu_start + (double)(ka + 2 * q) * a.dnu, nub = a.nu_start + (double)(kb + 2 * q) * a.dnu;
-          nuf[q] = make_float2((float)nua, (float)nub);
-          constexpr float C1 = (float)(2.0 * bartc::H * bartc::C * bartc::C);
-          c1nu3[q] = mul2(mul2(f2(C1), nuf[q]), mul2(nuf[q], nuf[q]));
-          // Rayleigh a nu^4 / (mu m_u) (in FP64: a / (mu m_u) may be below the FP32 range)
-          chi_r[q] = f2(0.0f);
-          if (a.ex.ray != 0.0)
-            chi_r[q] = make_float2((float)(a.ex.ray * (nua * nua) * (nua * nua)),
-                                   (float)(a.ex.ray * (nub * nub) * (nub * nub)));
+        const float2 nuf = make_float2((float)(a.nu_start + (double)ka * a.dnu), (float)(a.nu_start + (double)kb * a.dnu));
+        constexpr float C1 = (float)(2.0 * bartc::H * bartc::C * bartc::C);
+        const float2 c1nu3 = mul2(mul2(f2(C1), nuf), mul2(nuf, nuf));
+        // Rayleigh a nu^4 / (mu m_u) (in FP64: a / (mu m_u) may be below the FP32 range)
+        float2 chi_r = f2(0.0f);
+        if (a.ex.ray != 0.0) {
+          const double nua = a.nu_start + (double)ka * a.dnu, nub = a.nu_start + (double)kb * a.dnu;
+          chi_r = make_float2((float)(a.ex.ray * (nua * nua) * (nua * nua)), (float)(a.ex.ray * (nub * nub) * (nub * nub)));
         }
         const float* ga = a.grid + ka;
         const unsigned int dkb = (unsigned int)(kb - ka);
@@ -385,11 +380,11 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         // (tau the vertical optical depth from the top, ang_i = -log2(e)/mu_i)
         // only through their quadrature sum Tw = sum_i 2 pi w_i mu_i / 2 t_i,
         // so F = sum_k (B_{k-1} + B_k) (Tw_{k-1} - Tw_k) + 2 B_bottom Tw_bottom
-        float2 tau[P], Tw_prev[P], F[P], chi_prev[P], B_prev[P], B_hot[P];
+        float2 tau = f2(0.0f), Tw_prev = f2(a.tw_top), F = f2(0.0f);
         const int L_run = a.ex.L_run;
-        // grid values of a layer: lower (x) and upper (y) temperature bracket
-        // per species
-        auto fetch = [&](int k, float2 (*x)[P], float2 (*y)[P]) {
+        // grid values of a layer for both wavenumbers: lower (x) and upper (y)
+        // temperature bracket per species
+        auto fetch = [&](int k, float2* x, float2* y) {
           unsigned int of[4 * NCF];
 #pragma unroll
           for (int q = 0; q < NCF; ++q) {
@@ -401,23 +396,172 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           }
 #pragma unroll
           for (int q = 0; q < S; ++q) {
-            if (P == 2) {                          // ka is a multiple of 4 and ka + 3 < N here
-              const float4 u = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q]));
-              const float4 v = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q + 1]));
-              x[q][0] = make_float2(u.x, u.y);
-              x[q][P - 1] = make_float2(u.z, u.w);
-              y[q][0] = make_float2(v.x, v.y);
-              y[q][P - 1] = make_float2(v.z, v.w);
-            } else if (PAIR) {                     // ka is even and ka + 1 < N here
-              x[q][0] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q]));
-              y[q][0] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q + 1]));
+            if (PAIR) {                            // ka is even and ka + 1 < N here
+              x[q] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q]));
+              y[q] = __ldg(reinterpret_cast<const float2*>(ga + of[2 * q + 1]));
             } else {
-              x[q][0] = make_float2(__ldg(ga + of[2 * q]), __ldg(ga + (of[2 * q] + dkb)));
-              y[q][0] = make_float2(__ldg(ga + of[2 * q + 1]), __ldg(ga + (of[2 * q + 1] + dkb)));
+              x[q] = make_float2(__ldg(ga + of[2 * q]), __ldg(ga + (of[2 * q] + dkb)));
+              y[q] = make_float2(__ldg(ga + of[2 * q + 1]), __ldg(ga + (of[2 * q + 1] + dkb)));
             }
           }
         };
-        auto chi_of = [&](int k, const float2 (*x)[P], const float2 (*y)[P], float2* chi) {
+        auto chi_of = [&](int k, const float2* x, const float2* y) {
+          float cf[4 * NCF];
+#pragma unroll
+          for (int q = 0; q < NCF; ++q) {
+            const float4 v = s_rec[k].cf[q];
+            cf[4 * q] = v.x;
+            cf[4 * q + 1] = v.y;
+            cf[4 * q + 2] = v.z;
+            cf[4 * q + 3] = v.w;
+          }
+          float2 chi = chi_r;
+#pragma unroll
+          for (int q = 0; q < S; ++q) {
+            chi = fma2(f2(cf[2 * q]), x[q], chi);
+            chi = fma2(f2(cf[2 * q + 1]), y[q], chi);
+          }
+          return chi;
+        };
+        auto planck_k = [&](const float4& pl) {
+          if (WIDE_X) return planck2<true>(c1nu3, mul2(nuf, f2(pl.x)));
+          return planck_pair(c1nu3, nuf.x, pl.x, pl.z);
+        };
+        float2 cx[S], cy[S], nx[S], ny[S];
+        fetch(0, cx, cy);
+        fetch(min(1, L_run - 1), nx, ny);
+        float2 chi_prev = chi_of(0, cx, cy);
+        float2 B_prev = planck_k(s_rec[0].pl);
+        bool done_a = false, done_b = false;       // lane reached the optical-depth limit
+#pragma unroll 2
+        for (int k = 1; k < L_run; ++k) {
+#pragma unroll
+          for (int q = 0; q < S; ++q) {
+            cx[q] = nx[q];
+            cy[q] = ny[q];
+          }
+          fetch(min(k + 1, L_run - 1), nx, ny);    // the next layer's rows are in flight meanwhile
+          const float2 chi = chi_of(k, cx, cy);
+          const float4 pl = s_rec[k].pl;
+          const float2 B = planck_k(pl);
+          const float2 dtau = mul2(add2(chi_prev, chi), f2(pl.y));
+          const float2 Bsum = add2(B_prev, B);
+          tau = add2(tau, dtau);
+          float2 Tw0 = f2(0.0f), Tw1 = f2(0.0f);    // two partial sums: a shorter dependence chain
+#pragma unroll
+          for (int i = 0; i < NA; ++i) {
+            const float2 t = ex2_2(mul2(tau, f2(a.ang[i])));
+            if (i & 1) Tw1 = fma2(f2(a.ang[NA + i]), t, Tw1);
+            else Tw0 = fma2(f2(a.ang[NA + i]), t, Tw0);
+          }
+          const float2 Tw = add2(Tw0, Tw1);
+          const float2 Fn = fma2(Bsum, sub2(Tw_prev, Tw), F);
+          chi_prev = chi;
+          if (!TAU_LIM) {
+            F = Fn;
+            Tw_prev = Tw;
+            B_prev = B;
+          } else {
+            // Sec. 4 item 7: stop at the caller's optical-depth limit; the level
+            // reached is the bottom boundary (its blackbody below).  Each
+            // wavenumber of the pair keeps its state from the level where it
+            // stopped while the other goes on.
+            if (!done_a) {
+              F.x = Fn.x;
+              Tw_prev.x = Tw.x;
+              B_prev.x = B.x;
+            }
+            if (!done_b) {
+              F.y = Fn.y;
+              Tw_prev.y = Tw.y;
+              B_prev.y = B.y;
+            }
+            done_a = done_a || tau.x > a.ex.tau_cut;
+            done_b = done_b || tau.y > a.ex.tau_cut;
+            if (done_a && done_b) break;
+          }
+        }
+        F = fma2(mul2(f2(2.0f), B_prev), Tw_prev, F);   // the bottom level's blackbody through the column
+        if (a.spectra) {
+          const int64_t base = (a.offs ? a.offs[p] : (int64_t)p * a.N) - lo;
+          if (act_a) a.spectra[base + ja] = F.x;
+          if (act_b) a.spectra[base + jb] = F.y;
+        }
+
+        // 3. band sums of the tile, added to the unit's
+        if (nb > 0) {
+          const float dwa = act_a ? ((hi - lo == 1) ? 1.0f : ((ja == lo || ja == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
+          const float dwb = act_b ? ((hi - lo == 1) ? 1.0f : ((jb == lo || jb == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
+          const int warp = tid >> 5, lane = tid & 31;
+          for (int b = 0; b < nb; ++b) {
+            const float Wa = act_a ? __ldg(a.filt + (int64_t)b * a.N + ja) * dwa : 0.0f;
+            const float Wb = act_b ? __ldg(a.filt + (int64_t)b * a.N + jb) * dwb : 0.0f;
+            float num = fmaf(Wa, F.x, Wb * F.y), den = Wa + Wb;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              num += __shfl_xor_sync(0xffffffffu, num, o);
+              den += __shfl_xor_sync(0xffffffffu, den, o);
+            }
+            if (lane == 0) s_red[warp][b] = make_float2(num, den);
+          }
+          __syncthreads();
+          if (tid < nb) {
+#pragma unroll
+            for (int w = 0; w < NT / 32; ++w) {
+              band_acc.x += s_red[w][tid].x;
+              band_acc.y += s_red[w][tid].y;
+            }
+          }
+          __syncthreads();                         // s_red is rewritten by the next tile
+        }
+      };
+      // 2. two pairs a thread: the columns of wavenumbers ja .. ja + 3, read by
+      // one 16-byte load per row (a generic lambda: instantiated where it is used)
+      auto column4 = [&](auto, int tile) {
+        const int64_t ja = lo2 + (int64_t)tile * TW + 4 * tid;
+        const int64_t ka = (ja < hi) ? ja : lo2;   // idle lanes compute on valid indices
+        // the wavenumbers from their FP64 positions, the rest in FP32
+        float2 nuf[2], c1nu3[2], chi_r[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const double nua = a.nu_start + (double)(ka + 2 * q) * a.dnu;
+          const double nub = a.nu_start + (double)(ka + 2 * q + 1) * a.dnu;
+          nuf[q] = make_float2((float)nua, (float)nub);
+          constexpr float C1 = (float)(2.0 * bartc::H * bartc::C * bartc::C);
+          c1nu3[q] = mul2(mul2(f2(C1), nuf[q]), mul2(nuf[q], nuf[q]));
+          // Rayleigh a nu^4 / (mu m_u) (in FP64: a / (mu m_u) may be below the FP32 range)
+          chi_r[q] = f2(0.0f);
+          if (a.ex.ray != 0.0)
+            chi_r[q] = make_float2((float)(a.ex.ray * (nua * nua) * (nua * nua)),
+                                   (float)(a.ex.ray * (nub * nub) * (nub * nub)));
+        }
+        const float* ga = a.grid + ka;
+        float2 tau[2], Tw_prev[2], F[2], chi_prev[2], B_prev[2], B_hot[2];
+        const int L_run = a.ex.L_run;
+        // grid values of a layer: lower (x) and upper (y) temperature bracket
+        // per species
+        auto fetch = [&](int k, float2 (*x)[2], float2 (*y)[2]) {
+          unsigned int of[4 * NCF];
+#pragma unroll
+          for (int q = 0; q < NCF; ++q) {
+            const uint4 v = s_rec[k].off[q];
+            of[4 * q] = v.x;
+            of[4 * q + 1] = v.y;
+            of[4 * q + 2] = v.z;
+            of[4 * q + 3] = v.w;
+          }
+#pragma unroll
+          for (int q = 0; q < S; ++q) {
+            // ka is a multiple of 4 and ka + 3 < N here
+            const float4 u = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q]));
+            const float4 v = __ldg(reinterpret_cast<const float4*>(ga + of[2 * q + 1]));
+            x[q][0] = make_float2(u.x, u.y);
+            x[q][1] = make_float2(u.z, u.w);
+            y[q][0] = make_float2(v.x, v.y);
+            y[q][1] = make_float2(v.z, v.w);
+          }
+        };
+        auto chi_of = [&](int k, const float2 (*x)[2], const float2 (*y)[2], float2* chi) {
           float cf[4 * NCF];
 #pragma unroll
           for (int q = 0; q < NCF; ++q) {
@@ -428,7 +572,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
             cf[4 * q + 3] = v.w;
           }
 #pragma unroll
-          for (int i = 0; i < P; ++i) {
+          for (int i = 0; i < 2; ++i) {
             chi[i] = chi_r[i];
 #pragma unroll
             for (int q = 0; q < S; ++q) {
@@ -439,44 +583,34 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         };
         auto planck_k = [&](const float4& pl, float2* B) {
 #pragma unroll
-          for (int i = 0; i < P; ++i)
+          for (int i = 0; i < 2; ++i)
             B[i] = WIDE_X ? planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(pl.x))) : planck_pair(c1nu3[i], nuf[i].x, pl.x, pl.z);
         };
-        float2 cx[S][P], cy[S][P], nx[S][P], ny[S][P];
+        float2 cx[S][2], cy[S][2], nx[S][2], ny[S][2];
         fetch(0, cx, cy);
         fetch(min(1, L_run - 1), nx, ny);
         chi_of(0, cx, cy, chi_prev);
         planck_k(s_rec[0].pl, B_prev);
         const float y_hot = __int_as_float(s_ymin);
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
+        for (int i = 0; i < 2; ++i) {
           tau[i] = F[i] = f2(0.0f);
           Tw_prev[i] = f2(a.tw_top);
           // no level's Planck function is larger (up to rounding) than the hottest one's
           B_hot[i] = mul2(f2(2.0f / OPAQUE_SHARE), planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(y_hot))));
         }
-        bool done_a[P] = {}, done_b[P] = {};       // lane reached the optical-depth limit
+        bool done_a[2] = {}, done_b[2] = {};       // lane reached the optical-depth limit
         for (int k = 1; k < L_run;) {
-          const int k_look = P == 1 ? L_run : min(k + (TAU_LIM ? LOOK_EVERY_TAU_LIM : LOOK_EVERY), L_run);
+          const int k_look = min(k + (TAU_LIM ? LOOK_EVERY_TAU_LIM : LOOK_EVERY), L_run);
 #pragma unroll 2
           for (; k < k_look; ++k) {
-            float2 chi[P], B[P];
-            if (P == 1) {
-#pragma unroll
-              for (int q = 0; q < S; ++q) {
-                cx[q][0] = nx[q][0];
-                cy[q][0] = ny[q][0];
-              }
-              fetch(min(k + 1, L_run - 1), nx, ny);  // the next layer's rows are in flight meanwhile
-              chi_of(k, cx, cy, chi);
-            } else {                                 // one set of rows in registers
-              chi_of(k, nx, ny, chi);
-              fetch(min(k + 1, L_run - 1), nx, ny);
-            }
+            float2 chi[2], B[2];
+            chi_of(k, nx, ny, chi);                // one set of rows in registers
+            fetch(min(k + 1, L_run - 1), nx, ny);
             const float4 pl = s_rec[k].pl;
             planck_k(pl, B);
 #pragma unroll
-            for (int i = 0; i < P; ++i) {
+            for (int i = 0; i < 2; ++i) {
               tau[i] = add2(tau[i], mul2(add2(chi_prev[i], chi[i]), f2(pl.y)));
               chi_prev[i] = chi[i];
               const float2 Bsum = add2(B_prev[i], B[i]);
@@ -493,11 +627,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
                 F[i] = Fn;
                 Tw_prev[i] = Tw;
                 B_prev[i] = B[i];
-              } else {
-                // Sec. 4 item 7: stop at the caller's optical-depth limit; the level
-                // reached is the bottom boundary (its blackbody below).  Each
-                // wavenumber keeps its state from the level where it stopped
-                // while the others go on.
+              } else {                             // as with one pair
                 if (!done_a[i]) {
                   F[i].x = Fn.x;
                   Tw_prev[i].x = Tw.x;
@@ -512,27 +642,25 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
                 done_b[i] = done_b[i] || tau[i].y > a.ex.tau_cut;
               }
             }
-            if (P == 1 && TAU_LIM && done_a[0] && done_b[0]) break;
           }
-          if (P == 1) break;
           bool over = true;                          // (all lanes of a warp take the same levels)
 #pragma unroll
-          for (int i = 0; i < P; ++i) {
+          for (int i = 0; i < 2; ++i) {
             const float2 rest = mul2(B_hot[i], Tw_prev[i]);
             over = over && (done_a[i] || rest.x <= F[i].x) && (done_b[i] || rest.y <= F[i].y);
           }
           if (__all_sync(0xffffffffu, over)) break;
         }
         const int64_t base = a.spectra ? (a.offs ? a.offs[p] : (int64_t)p * a.N) - lo : 0;
-        float dw[2 * P], Fw[2 * P];                // trapezoid weights (0: not this span's), fluxes
+        float dw[4], Fw[4];                        // trapezoid weights (0: not this span's), fluxes
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
+        for (int i = 0; i < 2; ++i) {
           F[i] = fma2(mul2(f2(2.0f), B_prev[i]), Tw_prev[i], F[i]);   // the bottom level's blackbody through the column
           Fw[2 * i] = F[i].x;
           Fw[2 * i + 1] = F[i].y;
         }
 #pragma unroll
-        for (int i = 0; i < 2 * P; ++i) {
+        for (int i = 0; i < 4; ++i) {
           const int64_t j = ja + i;
           const bool act = j >= lo && j < hi;
           dw[i] = act ? ((hi - lo == 1) ? 1.0f : ((j == lo || j == hi - 1) ? 0.5f : 1.0f)) : 0.0f;
@@ -545,7 +673,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           for (int b = 0; b < nb; ++b) {
             float num = 0.0f, den = 0.0f;
 #pragma unroll
-            for (int i = 2 * P - 1; i >= 0; --i) {
+            for (int i = 3; i >= 0; --i) {
               const float Wi = dw[i] > 0.0f ? __ldg(a.filt + (int64_t)b * a.N + ja + i) * dw[i] : 0.0f;
               num = fmaf(Wi, Fw[i], num);
               den += Wi;
@@ -569,8 +697,9 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         }
       };
       for (int tile = grp * a.tpu; tile < t_end; ++tile) {
-        if (P == 2 || pair_loads) column(std::true_type{}, tile);
-        else if (P == 1) column(std::integral_constant<bool, P == 2>{}, tile);   // (only P = 1 has the form)
+        if constexpr (P == 2) column4(0, tile);
+        else if (pair_loads) column(std::true_type{}, tile);
+        else column(std::false_type{}, tile);
       }
 
       // the unit's band partials; the proposal's last unit reduces them
