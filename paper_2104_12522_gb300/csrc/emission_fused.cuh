@@ -1083,6 +1083,7 @@ cudaError_t launch_pair(const FusedArgs& a, int sm_count, cudaStream_t st) {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, emission_fused_kernel<S, NA, NT, P, MODE>, NT, 0);
   if (e != cudaSuccess) return e;
   unsigned long long grid = (unsigned long long)(per_sm < 1 ? 1 : per_sm) * (unsigned long long)sm_count;
+  if (a.n_units == 0) return cudaSuccess;          // the kernel is loaded by now, which is all the call is for
   if (grid > a.n_units) grid = a.n_units;
   emission_fused_kernel<S, NA, NT, P, MODE><<<(unsigned)grid, NT, 0, st>>>(a);
   return cudaGetLastError();
@@ -1098,6 +1099,7 @@ cudaError_t launch_tma(const FusedArgs& a, int sm_count, cudaStream_t st) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, emission_tma_kernel<S, NA, TW>, TW / 2 + 32, smem);
   if (e != cudaSuccess) return e;
   unsigned long long grid = (unsigned long long)(per_sm < 1 ? 1 : per_sm) * (unsigned long long)sm_count;
+  if (a.n_units == 0) return cudaSuccess;          // the kernel is loaded by now, which is all the call is for
   if (grid > a.n_units) grid = a.n_units;
   emission_tma_kernel<S, NA, TW><<<(unsigned)grid, TW / 2 + 32, smem, st>>>(a);
   return cudaGetLastError();

@@ -125,7 +125,7 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   }
   const long long span_cap =
       (l2_bytes > 0 ? (long long)l2_bytes / 2 : (64LL << 20)) / ((long long)S * L * M * (long long)sizeof(float));
-  auto run = [&](int nt) -> bart_status {
+  auto run = [&](int nt, bool load_only = false) -> bart_status {
     const int tw = fused_width(form, nt);
     // several consecutive tiles per unit amortise the unit's fixed work (layer
     // states, band partials and counts), as long as there are enough units to
@@ -135,7 +135,7 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
     const long long tpu_cap = std::max(1LL, std::min<long long>(MAX_TILES_PER_UNIT, span_cap / tw));
     a.tpu = (int)std::max(1LL, std::min<long long>(tpu_cap, (long long)n * n_tiles / target));
     a.n_groups = (n_tiles + a.tpu - 1) / a.tpu;
-    a.n_units = (unsigned long long)a.n_groups * (unsigned long long)n;
+    a.n_units = load_only ? 0 : (unsigned long long)a.n_groups * (unsigned long long)n;
     cudaError_t e = pick_fused(S, NA, form, nt, mode)(a, ctx->sm_count, ctx->stream);
     if (e != cudaSuccess) return bart_fail(ctx, BART_ECUDA, "launch of emission_fused_kernel failed: %s",
                                            cudaGetErrorString(e));
@@ -153,6 +153,11 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
     // fixed by the caller
   } else if (it != ctx->tiles.end()) {
     nt = it->second / fused_width(form, 1);
+  } else if (ctx->autotune && (long long)n * max_tiles <= 2LL * ctx->sm_count) {
+    // At most about a unit per SM: the widths run alike (31.8, 31.7 and 31.9 us
+    // for one spectrum of 2,000 points at 64, 128 and 256 threads), below what
+    // one run of each can tell.
+    ctx->tiles[key] = fused_width(form, nt);
   } else if (ctx->autotune) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     BART_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cs));
@@ -161,6 +166,12 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
       BART_CUDA(ctx, cudaEventCreate(&e0));
       BART_CUDA(ctx, cudaEventCreate(&e1));
       float best = 1e30f;
+      // Each candidate is another kernel, which the driver loads at its first
+      // use: here, before the timing, where it decided the choice by chance (301
+      // ragged spectra took 256 threads in one of six programs, 674 us for 648 at
+      // 128).
+      for (int cand : FUSED_THREADS)
+        if ((st = run(cand, true)) != BART_OK) return st;
       for (int cand : FUSED_THREADS) {
         BART_CUDA(ctx, cudaEventRecord(e0, ctx->stream));
         if ((st = run(cand)) != BART_OK) return st;
