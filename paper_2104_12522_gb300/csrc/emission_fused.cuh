@@ -674,7 +674,9 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
             float num = 0.0f, den = 0.0f;
 #pragma unroll
             for (int i = 3; i >= 0; --i) {
-              const float Wi = dw[i] > 0.0f ? __ldg(a.filt + (int64_t)b * a.N + ja + i) * dw[i] : 0.0f;
+              // (what lies outside the span may not be finite: left out, not multiplied by 0)
+              if (dw[i] == 0.0f) continue;
+              const float Wi = __ldg(a.filt + (int64_t)b * a.N + ja + i) * dw[i];
               num = fmaf(Wi, Fw[i], num);
               den += Wi;
             }
