@@ -255,6 +255,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
   __shared__ LayerRec<S> s_rec[MAX_LAYERS];
   __shared__ float s_xs[S];
   __shared__ float2 s_red[NT / 32 > 0 ? NT / 32 : 1][MAX_BANDS];
+  __shared__ double2 s_band[P == 2 ? MAX_BANDS : 1];   // two pairs: a unit's band sums (no registers left for them)
   __shared__ unsigned long long s_unit;
   __shared__ int s_last, s_ready, s_ymin;
   constexpr bool WIDE_X = (MODE & 1) != 0, TAU_LIM = (MODE & 2) != 0;
@@ -353,7 +354,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
       }
       __syncthreads();
       if (!ready && tid == 0) st_release(a.tw_flag + p, ready_mark);   // publishes the CTA's stores above
-      float2 band_acc = make_float2(0.f, 0.f);      // thread b < nb: band b over the unit's tiles
+      float band_num = 0.0f, band_den = 0.0f;       // one pair: thread b < nb, band b over the unit's tiles
+      if (P == 2 && tid < nb) s_band[tid] = make_double2(0.0, 0.0);
       const int t_end = min((grp + 1) * a.tpu, n_tiles_p);
 
       // 2. one pair a thread: the columns of wavenumbers ja and ja + 1 of one
@@ -508,8 +510,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           if (tid < nb) {
 #pragma unroll
             for (int w = 0; w < NT / 32; ++w) {
-              band_acc.x += s_red[w][tid].x;
-              band_acc.y += s_red[w][tid].y;
+              band_num += s_red[w][tid].x;
+              band_den += s_red[w][tid].y;
             }
           }
           __syncthreads();                         // s_red is rewritten by the next tile
@@ -670,6 +672,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
         // 3. band sums of the tile, added to the unit's
         if (nb > 0) {
           const int warp = tid >> 5, lane = tid & 31;
+          // (units are twice as wide as with one pair: the warps' sums are added
+          // as a tree and the tiles' in FP64, so that the bands round no more)
           for (int b = 0; b < nb; ++b) {
             float num = 0.0f, den = 0.0f;
 #pragma unroll
@@ -689,11 +693,15 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           }
           __syncthreads();
           if (tid < nb) {
+            float2 w[NT / 32];
 #pragma unroll
-            for (int w = 0; w < NT / 32; ++w) {
-              band_acc.x += s_red[w][tid].x;
-              band_acc.y += s_red[w][tid].y;
-            }
+            for (int q = 0; q < NT / 32; ++q) w[q] = s_red[q][tid];
+#pragma unroll
+            for (int o = NT / 64; o > 0; o >>= 1)
+#pragma unroll
+              for (int q = 0; q < o; ++q) w[q] = add2(w[q], w[q + o]);
+            s_band[tid].x += w[0].x;
+            s_band[tid].y += w[0].y;
           }
           __syncthreads();                         // s_red is rewritten by the next tile
         }
@@ -706,7 +714,9 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
 
       // the unit's band partials; the proposal's last unit reduces them
       if (nb > 0) {
-        if (tid < nb) a.partial[((int64_t)p * a.n_groups + grp) * nb + tid] = band_acc;
+        if (tid < nb)
+          a.partial[((int64_t)p * a.n_groups + grp) * nb + tid] =
+              P == 2 ? make_float2((float)s_band[tid].x, (float)s_band[tid].y) : make_float2(band_num, band_den);
         __syncthreads();
         if (tid == 0) s_last = (add_acq_rel(a.p_done + p, 1u) + 1u == (unsigned)n_groups_p);
         __syncthreads();
