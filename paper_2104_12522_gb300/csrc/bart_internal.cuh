@@ -35,6 +35,7 @@ struct bart_ctx {
   int em_tile = 0;                  // emission tile width fixed by the caller (0: autotuner)
   int em_launch = BART_LAUNCH_FUSED; // emission launch structure (bart_set_emission_launch)
   cudaStream_t user_stream = nullptr;  // the caller's stream while a capture is open
+  const int* grid_bad = nullptr;    // what bart_retrieval_run found of its grid (bartem::check_grid_values), while it runs
   bool own_capture = false;         // the capture of bart_retrieval_run, whose graph ends with the call
   bool capturing = false;           // between bart_capture_begin and bart_capture_end
   int* d_status = nullptr;          // device status word

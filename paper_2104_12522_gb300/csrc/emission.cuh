@@ -113,6 +113,14 @@ struct EmPrep {
 bart_status emission_prologue(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
                               EmPrep* out, int* zero = nullptr, size_t zero_words = 0);
 
+// Whether a (valid) call's columns may end early once the grid's values are
+// known to be finite and not negative: two pairs a thread, no spans (which may
+// leave most of the grid unread), no negative abundance.
+bool columns_may_end(const bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b);
+// Launches the check of them; *bad: device word, 0 where they are
+// (forward_fused.cu).
+bart_status check_grid_values(bart_ctx* ctx, const bart_grid_desc* g, const int** bad);
+
 // The persistent fused launch of an emission batch (forward_fused.cu).
 bart_status fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b,
                            float* spectra, const bart_filters* f, float* bands, int nb);

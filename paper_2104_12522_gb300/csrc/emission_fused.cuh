@@ -114,16 +114,20 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned i
 
 // With two pairs a thread, a warp's column ends where twice the largest Planck
 // function of the profile times the transmittance left is below this share of
-// the flux gathered so far at every wavenumber: what lies below adds at most
-// that (the layers' terms telescope), a quarter of the flux's rounding.  The
-// rows below are not read, which is the point: 2,048 proposals on the 100-layer
-// grid read 655 GB from L2 if they read every layer (18 TB/s at 36.3 ms), and
-// 36% of the layers of prior draws lie below.
+// the flux gathered so far at every wavenumber: no layer below adds as much as
+// half a unit in the last place of the flux, so the sum over all layers gives
+// the same bits.  That holds for opacities that are finite and not negative,
+// which grid_check_kernel establishes (a NaN below an opaque level reaches the
+// spectrum as from any other); columns of other grids, and of calls that are
+// too small for the check to pay, take every layer.  The rows below are not
+// read, which is the point: 2,048 proposals on the 100-layer grid read 655 GB
+// from L2 if they read every layer (18 TB/s at 36.3 ms), and 36% of the layers
+// of prior draws lie below.
 constexpr float OPAQUE_SHARE = 1.0f / (float)(1 << 26);
 // Levels between two looks; two with the optical-depth limit, which ends
 // columns by the same test.  2,048 proposals: 36.3 ms with one pair and no
-// looks, 33.6 with two pairs, 28.0-28.6 with looks (29-30 with looks inside the level
-// loop).  One pair a thread (30.9 ms with looks) takes none: its looks cost 8%
+// looks, 33.6 with two pairs, 27.9 with looks (29-30 with looks inside the level
+// loop), 28.4 with the check of the grid.  One pair a thread (30.9 ms with looks) takes none: its looks cost 8%
 // of 301 ragged spectra on odd rows down to a cloud deck (642 us), where few
 // columns end early.
 constexpr int LOOK_EVERY = 8, LOOK_EVERY_TAU_LIM = 2;
@@ -162,6 +166,7 @@ struct FusedArgs {
   unsigned int* tw_flag;             // [n] epoch + 1 once tw_cache[p] holds this launch's states
   int* status;
   EmExtra ex;
+  const int* grid_bad;               // device word: 0 where every opacity is finite and not negative; NULL: not known
   bool wide_x;                       // c2 nu / T can exceed 20: FP64 Planck branch
   bool tau_lim;                      // the optical-depth limit is on
 };
@@ -257,7 +262,7 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
   __shared__ float2 s_red[NT / 32 > 0 ? NT / 32 : 1][MAX_BANDS];
   __shared__ double2 s_band[P == 2 ? MAX_BANDS : 1];   // two pairs: a unit's band sums (no registers left for them)
   __shared__ unsigned long long s_unit;
-  __shared__ int s_last, s_ready, s_ymin;
+  __shared__ int s_last, s_ready, s_ymin, s_ends;
   constexpr bool WIDE_X = (MODE & 1) != 0, TAU_LIM = (MODE & 2) != 0;
   const int tid = threadIdx.x;
   const int L = a.L, nb = a.n_bands;
@@ -306,13 +311,17 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
       // others (a unit that finds them unpublished computes them itself),
       // and from them the layer records
       if (tid == 0) s_ready = (ld_acquire(a.tw_flag + p) == ready_mark);
-      if (P == 2 && tid == 0) s_ymin = 0x7f800000;
+      if (P == 2 && tid == 0) {
+        s_ymin = 0x7f800000;
+        s_ends = a.grid_bad && *a.grid_bad == 0;   // columns may end early (OPAQUE_SHARE)
+      }
       if (tid < S) {
         const float ab = a.theta ? a.theta[(int64_t)p * a.n_theta + 5 + tid] : 0.0f;
         s_xs[tid] = a.x0mu[tid] * exp10f(ab);
       }
       __syncthreads();
       const bool ready = s_ready;
+      if (P == 2 && tid < S && !(s_xs[tid] <= 3.402823466e38f)) s_ends = 0;
       for (int k = tid; k < L; k += NT) {
         LayerTW r;
         if (ready) {
@@ -599,7 +608,8 @@ emission_fused_kernel(const __grid_constant__ FusedArgs a) {
           tau[i] = F[i] = f2(0.0f);
           Tw_prev[i] = f2(a.tw_top);
           // no level's Planck function is larger (up to rounding) than the hottest one's
-          B_hot[i] = mul2(f2(2.0f / OPAQUE_SHARE), planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(y_hot))));
+          // (infinite where columns may not end: no test passes then)
+          B_hot[i] = mul2(f2(s_ends ? 2.0f / OPAQUE_SHARE : INFINITY), planck2<WIDE_X>(c1nu3[i], mul2(nuf[i], f2(y_hot))));
         }
         bool done_a[2] = {}, done_b[2] = {};       // lane reached the optical-depth limit
         for (int k = 1; k < L_run;) {

@@ -24,24 +24,83 @@ FusedLauncher pick_fused(int S, int na, FusedForm form, int nt, int mode) {
   }
 }
 
+// The form of a call of n proposals: the bulk-copy variant on request, where
+// its 16-byte row starts hold (n_nu a multiple of 4 and an aligned grid), else two
+// pairs per thread where the rows allow it and the call has enough wavenumbers
+// to fill the SMs twice with such threads (354 proposals on 1,600, a fill and a
+// half: 80 us in pairs, 84 with two), from 24 proposals on or where columns may
+// end early.  Without early ends, on the 100-layer grid of 4 species: 16
+// proposals 410 us in pairs and 417 with two (few share a row: DRAM), 32 716 and
+// 688, 512 9.30 and 8.65 ms; with them 512 7.60 ms, 16 of a checked grid 328 us.
+FusedForm fused_form(const bart_ctx* ctx, const bart_grid_desc* g, int n, bool ends) {
+  const int64_t N = g->nu.n_nu;
+  const bool rows16 = (N % 4 == 0) && (reinterpret_cast<uintptr_t>(g->grid) % 16 == 0);
+  return !rows16 ? FUSED_PAIR
+         : ctx->em_launch == BART_LAUNCH_FUSED_TMA ? FUSED_BULK
+         : (n >= 24 || ends) && (double)n * (double)N >= 8.0 * FUSED_OCC_THREADS2 * ctx->sm_count ? FUSED_TWO_PAIRS
+                                                                                                  : FUSED_PAIR;
+}
+
+// Sets *bad where a value of the grid is negative (or -0), infinite or not a
+// number: its bits are above those of the largest float.  Bound by the reads of
+// the grid from DRAM.
+constexpr int CHECK_THREADS = 512;
+__global__ void __launch_bounds__(CHECK_THREADS)
+grid_check_kernel(const float* __restrict__ grid, size_t n, int* __restrict__ bad) {
+  const size_t step = (size_t)gridDim.x * CHECK_THREADS, first = (size_t)blockIdx.x * CHECK_THREADS + threadIdx.x;
+  unsigned int m = 0;
+  if ((reinterpret_cast<uintptr_t>(grid) & 15) == 0) {
+    const uint4* g4 = reinterpret_cast<const uint4*>(grid);
+#pragma unroll 8
+    for (size_t i = first; i < n / 4; i += step) {
+      const uint4 v = __ldg(g4 + i);
+      m = max(max(max(m, v.x), max(v.y, v.z)), v.w);
+    }
+    for (size_t i = n / 4 * 4 + first; i < n; i += step) m = max(m, __float_as_uint(__ldg(grid + i)));
+  } else {
+    for (size_t i = first; i < n; i += step) m = max(m, __float_as_uint(__ldg(grid + i)));
+  }
+  if (m > 0x7f7fffffu) *bad = 1;
+}
+
+// Proposals per grid temperature from which a call checks the grid so that
+// columns may end early.  The check reads S L M n_nu values from DRAM (3.2 GB:
+// 0.48 ms); the layers that n proposals leave out save 0.40 ms of 128 proposals
+// on a grid of 20 temperatures, 0.78 ms of 256, 1.5 ms of 512.
+constexpr int CHECK_FROM = 10;
+
 }  // namespace
+
+bool bartem::columns_may_end(const bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c, const bart_batch* b) {
+  bool ends = ctx->em_launch != BART_LAUNCH_SPLIT && fused_offsets_fit(g) &&
+              fused_form(ctx, g, b->n, true) == FUSED_TWO_PAIRS && !b->nu_lo;
+  for (int s = 0; s < g->n_species; ++s) ends = ends && c->x0[s] >= 0.0;
+  return ends;
+}
+
+bart_status bartem::check_grid_values(bart_ctx* ctx, const bart_grid_desc* g, const int** bad) {
+  void* p = nullptr;
+  bart_status st;
+  if ((st = bart_scratch(ctx, "ff_bad", sizeof(int), &p)) != BART_OK) return st;
+  BART_CUDA(ctx, cudaMemsetAsync(p, 0, sizeof(int), ctx->stream));
+  const size_t n = (size_t)g->n_species * g->n_layers * g->n_temps * (size_t)g->nu.n_nu;
+  const size_t want = n / (32 * CHECK_THREADS) + 1;      // 8 16-byte loads a thread
+  grid_check_kernel<<<(unsigned)std::min<size_t>(want, 4 * (size_t)ctx->sm_count), CHECK_THREADS, 0, ctx->stream>>>(
+      g->grid, n, (int*)p);
+  *bad = (const int*)p;
+  return bart_check_launch(ctx, "grid_check_kernel");
+}
 
 bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const bart_fwd_cfg* c,
                                    const bart_batch* b, float* spectra, const bart_filters* f, float* bands, int nb) {
   const int S = g->n_species, L = g->n_layers, M = g->n_temps, n = b->n, NA = c->n_angles;
   const int64_t N = g->nu.n_nu;
   const int mode = emission_mode(g, c);
-  // the bulk-copy variant on request, where its 16-byte row starts hold:
-  // n_nu a multiple of 4 and an aligned grid
-  const bool rows16 = (N % 4 == 0) && (reinterpret_cast<uintptr_t>(g->grid) % 16 == 0);
-  // else two pairs per thread where the rows allow it and the call has enough
-  // wavenumbers to fill the SMs twice with such threads (16 proposals on 100,000
-  // wavenumbers: 418 us in pairs, 370 with two; 354 on 1,600, a fill and a half:
-  // 80 us in pairs, 84 with two)
-  const FusedForm form = !rows16 ? FUSED_PAIR
-                         : ctx->em_launch == BART_LAUNCH_FUSED_TMA ? FUSED_BULK
-                         : (double)n * (double)N >= 8.0 * FUSED_OCC_THREADS2 * ctx->sm_count ? FUSED_TWO_PAIRS
-                                                                                            : FUSED_PAIR;
+  // columns may end early where the grid was checked (by the retrieval loop) or
+  // the check pays for the call (of which every proposal is active)
+  const bool ends =
+      (ctx->grid_bad || (n >= (int64_t)CHECK_FROM * M && !b->active)) && columns_may_end(ctx, g, c, b);
+  const FusedForm form = fused_form(ctx, g, n, ends);
   if (S > FUSED_MAX_SPECIES || !pick_fused(S, NA, form, FUSED_THREADS[1], mode))
     return bart_fail(ctx, BART_EUNSUPPORTED, "emission with %d species and %d angles is not instantiated "
                      "(species 1-4; angles 1, 2, 4, 8, 16)", S, NA);
@@ -111,6 +170,8 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   a.tw_flag = (unsigned int*)p_flag;
   a.status = ctx->d_status;
   a.ex = emission_extra(g, c);
+  if (ends && ctx->grid_bad) a.grid_bad = ctx->grid_bad;
+  else if (ends && (st = check_grid_values(ctx, g, &a.grid_bad)) != BART_OK) return st;
   a.wide_x = (mode & 1) != 0;
   a.tau_lim = (mode & 2) != 0;
 
@@ -144,8 +205,8 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   // threads per CTA: fixed by the caller, cached per shape, or measured once
   // (each candidate timed with CUDA events on the stream) outside a capture
   char key[160];
-  snprintf(key, sizeof(key), "fused%s S%d A%d L%d/%d M%d N%lld n%d b%d span%d m%d", form == FUSED_BULK ? " tma" : form == FUSED_TWO_PAIRS ? " x4" : "", S, NA, L,
-           a.ex.L_run, M, (long long)N, n, nb, b->nu_lo ? 1 : 0, mode);
+  snprintf(key, sizeof(key), "fused%s S%d A%d L%d/%d M%d N%lld n%d b%d span%d m%d", form == FUSED_BULK ? " tma" : ends ? " x4 ends" : form == FUSED_TWO_PAIRS ? " x4" : "",
+           S, NA, L, a.ex.L_run, M, (long long)N, n, nb, b->nu_lo ? 1 : 0, mode);
   // (the caller's width is that of the one-wavenumber-per-thread kernels)
   int nt = ctx->em_tile > 0 ? ctx->em_tile : FUSED_THREADS[1];
   auto it = ctx->tiles.find(key);

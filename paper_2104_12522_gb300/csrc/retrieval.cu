@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "demc.cuh"
+#include "emission.cuh"
 
 namespace {
 
@@ -93,7 +94,17 @@ extern "C" bart_status bart_retrieval_run(bart_ctx* ctx, bart_demc* s, bart_mlp*
     return BART_OK;
   };
 
-  r = generation();           // eager: sizes scratch, uploads constants
+  // One check of the grid for all generations, which lets the emission columns
+  // end early: some proposals are screened out, so from twice the proposals on
+  // that a single call asks.  (What is not valid is left to the forward model.)
+  struct Checked {
+    bart_ctx* ctx;
+    ~Checked() { ctx->grid_bad = nullptr; }
+  } checked{ctx};
+  if ((double)C * n_generations >= 32.0 * grid->n_temps &&
+      bartem::check_forward_request(ctx, grid, cfg, &batch) == BART_OK && bartem::columns_may_end(ctx, grid, cfg, &batch))
+    r = bartem::check_grid_values(ctx, grid, &ctx->grid_bad);
+  if (r == BART_OK) r = generation();           // eager: sizes scratch, uploads constants
   if (r == BART_OK && n_generations > 1) {
     if (use_graph) {
       // Capture on a private non-blocking stream ordered after the caller's
