@@ -362,9 +362,7 @@ typedef struct {
  *   filters  bands to integrate, or NULL
  *   bands    device [n][filters->n_bands] or NULL (needs filters)
  * Band values are the trapezoid-weighted means of bart_band_integrate; a band
- * with no weight on an entry's span yields 0.  Opacities are finite and not
- * negative; below levels that are opaque at FP32 they may stay unread.  An
- * entry whose span is invalid
+ * with no weight on an entry's span yields 0.  An entry whose span is invalid
  * (lo < 0, hi > nu.n_nu or lo >= hi) keeps its spectrum untouched, gets band
  * values 0 and makes bart_sync() return BART_ERANGE. */
 bart_status bart_forward_spectra_batch(bart_ctx* ctx, const bart_grid_desc* grid,

@@ -402,7 +402,9 @@ trans_kernel(const float* __restrict__ grid, int Lg, int M, int64_t N, const TrL
     // A ray's longest chords lie in the shells next to its lowest point: those
     // of the last TR_TAIL shells of a block are summed first.  Where they alone
     // make every ray of the block opaque over the warp (1 - e^-tau is 1 in
-    // FP32) the shells above change nothing and are left out.
+    // FP32) the shells above change nothing and are left out.  (Every shell is
+    // among the last TR_TAIL of some block, whose rays' paths through it are the
+    // longest: a NaN reaches the spectrum from any of them.)
     auto tail = [&](const float* d, int k0, int k1, float2* t) {
 #pragma unroll
       for (int r = 0; r < TR_RB; ++r) t[r] = tr_f2(0.f);
