@@ -21,10 +21,11 @@
 // row over the whole grid for every band.  They are now taken over each
 // filter's extent only, in pairs of FP32 (two-sum and two-product: the sums
 // carry about 48 bits, the band value is FP32), with a band's weights read
-// once for 8 rows.
+// once for 8 rows.  The terms of deep rows go down to FP32's smallest numbers, so
+// they are scaled for the products (CB_SCALE).
 // Measured, 4 proposals x 100 layers x 100,000 wavenumbers, 4 species, 10
-// bands: 3.47 ms before, 0.45 ms
-// now; the rows' reads alone need 0.19 ms of the DRAM copy rate.
+// bands: 3.47 ms before, 0.38 ms now (0.59 ms with every sum in FP64); the rows'
+// reads alone need 0.19 ms of the DRAM copy rate.
 #include <algorithm>
 #include <cmath>
 
@@ -219,6 +220,15 @@ contrib_kernel(const float* __restrict__ grid, int L, int M, int64_t N, const La
   for (int q = k; q < L; ++q) store(q, f2(0.0f));
 }
 
+// The terms are multiplied by CB_SCALE (exactly) before their products with the
+// weights, so that no product's low part that matters lies below the FP32 range:
+// what 2^17 products lose there, 2^-149 each, is 2^-188 of a band's sum, for
+// weights that sum to CB_LEAST 2^-175 of its value, below 2^-26 of the smallest
+// FP32 number.  Sums that are larger than CB_MOST or not finite, and smaller weights, are
+// taken again in FP64.
+constexpr float CB_SCALE = 7.205759403792794e16f;                                   // 2^56
+constexpr double CB_LEAST = 1.220703125e-4, CB_MOST = 1.329227995784916e36;         // 2^-13, 2^120
+
 // Band means of CB_ROWS contribution rows of one proposal: trapezoid weights
 // over the proposal's span, the sums as FP32 pairs per thread and across the
 // warp, FP64 across the warps.
@@ -246,7 +256,7 @@ contrib_band_kernel(const float* __restrict__ contrib, int L, int64_t N, const i
     const float W = __ldg(w + j) * dw;         // exact: dw is 1 or 1/2
     pair_add(den, W, 0.0f);
 #pragma unroll
-    for (int r = 0; r < CB_ROWS; ++r) pair_fma(num[r], W, __ldg(c[r] + j));
+    for (int r = 0; r < CB_ROWS; ++r) pair_fma(num[r], W, __ldg(c[r] + j) * CB_SCALE);
   }
   __shared__ double sh[CB_THREADS / 32][CB_ROWS + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -257,23 +267,45 @@ contrib_band_kernel(const float* __restrict__ contrib, int L, int64_t N, const i
       pair_add(v, h, 0.0f);
       v.lo += l;
     }
-    if (lane == 0) {
-      // where hi is not finite the pair's lo is NaN: the sum is hi itself
-      sh[warp][slot] = fabsf(v.hi) <= 3.402823466e38f ? (double)v.hi + (double)v.lo : (double)v.hi;
-    }
+    if (lane == 0) sh[warp][slot] = (double)v.hi + (double)v.lo;
   };
 #pragma unroll
   for (int r = 0; r < CB_ROWS; ++r) reduce(num[r], r);
   reduce(den, CB_ROWS);
   __syncthreads();
-  if ((int)threadIdx.x < nr) {
-    double a = 0.0, d = 0.0;
+  double a = 0.0, d = 0.0;
+  auto add = [&]() {
+    a = d = 0.0;
     for (int q = 0; q < CB_THREADS / 32; ++q) {
-      a += sh[q][threadIdx.x];
+      a += sh[q][min((int)threadIdx.x, CB_ROWS)];
       d += sh[q][CB_ROWS];
     }
-    out[((int64_t)p * L + k0 + threadIdx.x) * n_bands + b] = d > 0.0 ? (float)(a / d) : 0.0f;
+  };
+  add();
+  if (__syncthreads_or((int)threadIdx.x < nr && !(fabs(a) <= CB_MOST && d >= CB_LEAST && d <= CB_MOST))) {
+    double sum[CB_ROWS] = {}, weight = 0.0;    // the products of FP32 values are exact
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += CB_THREADS) {
+      const float dw = (hi - lo == 1) ? 1.0f : ((j == lo || j == hi - 1) ? 0.5f : 1.0f);
+      const double W = (double)(__ldg(w + j) * dw);
+      weight += W;
+#pragma unroll
+      for (int r = 0; r < CB_ROWS; ++r) sum[r] = fma(W, (double)__ldg(c[r] + j), sum[r]);
+    }
+    auto put = [&](double v, int slot) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) sh[warp][slot] = v;
+    };
+#pragma unroll
+    for (int r = 0; r < CB_ROWS; ++r) put(sum[r], r);
+    put(weight, CB_ROWS);
+    __syncthreads();
+    add();
+  } else {
+    a *= 1.0 / (double)CB_SCALE;
   }
+  if ((int)threadIdx.x < nr)
+    out[((int64_t)p * L + k0 + threadIdx.x) * n_bands + b] = d > 0.0 ? (float)(a / d) : 0.0f;
 }
 
 using CfLauncher = void (*)(dim3, cudaStream_t, const float*, int, int, int64_t, const LayerTW*, const float*,
