@@ -20,9 +20,10 @@
 // series of the Voigt profile and the expansion about the centre in one).  The
 // E[z^n] follow K_0 = 1, K_1 = w, K_(n+1) = w K_n + n sigma^2 K_(n-1),
 // w = delta + i gamma; a block keeps I_n = sum_lines (S / pi) Im K_n, n = 1 ..
-// DN_P.  m1 and m2 keep sqrt(half^2 + gamma^2) <= DN_RHO x the distance: the
-// first term left out is then below 9 DN_RHO^8 = 1.3e-6 of a line's own at the
-// nearest point for the line farthest from the centre, far below that in a sum.
+// DN_P.  m1 and m2 keep sqrt(r^2 + gamma^2) <= DN_RHO x the distance, r^8 =
+// E[(half + g)^8] (reach8): the first term left out is then below 9 DN_RHO^8 =
+// 1.3e-6 of a line's own at the nearest point for the line farthest from the
+// centre, far below that in a sum.
 //
 // Lengths are in units of a power of two near the widest profile, so that no
 // power of a width leaves the FP32 range.
@@ -32,7 +33,9 @@
 // u = delta + g + i (gamma - gamma_c) about the bin's middle gamma_c and
 // Z = d - i gamma_c, V = (S / pi) Im sum_n E[u^n] / Z^(n+1): |Z| >= gamma_c, so a
 // wide profile is smooth on the scale of a block and needs no near lines at
-// all.  DN_PC terms hold where |u| <= DN_RHOC |Z| (15 DN_RHOC^14 = 9e-7).
+// all.  DN_PC terms hold where E[|u|^14] <= (DN_RHOC |Z|)^14 (reach14; 15
+// DN_RHOC^14 = 9e-7; against the Faddeeva function in 64 bits, for x of a grid
+// interval from 0.4 on: 1.2e-6 of a line on its block's edge).
 // Distances where the moments about the real centre hold take those (one set
 // per block, half the operations).
 //
@@ -259,8 +262,26 @@ __device__ DenseBins dense_bins(const int* __restrict__ stat) {
   return r;
 }
 
+// (E[(h + g)^8])^(1/8) and (E[(h + g)^14])^(1/14) of a Gaussian g of deviation s:
+// how far a line h from its block's centre reaches into the moments.
+__device__ __forceinline__ float reach8(float h, float s) {
+  const float r = s / h, q = r * r;
+  return h * powf(fmaf(q, fmaf(q, fmaf(q, fmaf(q, 105.0f, 420.0f), 210.0f), 28.0f), 1.0f), 0.125f);
+}
+__device__ __forceinline__ float reach14(float h, float s) {
+  const float r = s / h, q = r * r;
+  float v = fmaf(q, 135135.0f, 945945.0f);
+  v = fmaf(q, v, 945945.0f);
+  v = fmaf(q, v, 315315.0f);
+  v = fmaf(q, v, 45045.0f);
+  v = fmaf(q, v, 3003.0f);
+  v = fmaf(q, v, 91.0f);
+  return h * powf(fmaf(q, v, 1.0f), 1.0f / 14.0f);
+}
+
+// sigma: the widest Doppler deviation of a cell in points, over dfac.
 __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cells, const int* __restrict__ stat,
-                                  float inv_dnu, int reach, DensePlan* __restrict__ plan,
+                                  float inv_dnu, float sigma, int reach, DensePlan* __restrict__ plan,
                                   DenseBins* __restrict__ bins) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const DenseBins bn = dense_bins(stat);
@@ -270,8 +291,10 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
   const float scale = cells[c].gfac * inv_dnu, g = __int_as_float(stat[0]) * scale;   // widest line, in points
   if (cells[c].dense && !stat[1] && g < 1e6f) {
     // a point of block t is at least 8 m - 3.5 points from the centre of block t +- m
-    const int m1 = max(DN_M1, (int)ceilf((sqrtf(16.0f + g * g) / DN_RHO + 3.5f) / 8.0f));
-    const int m2 = max(4, (int)ceilf((sqrtf(256.0f + g * g) / DN_RHO + 15.5f) / 32.0f));
+    const float sd = sigma * cells[c].dfac;
+    const float r8 = reach8(4.0f, sd), r32 = reach8(16.0f, sd), c8 = reach14(4.0f, sd), c32 = reach14(16.0f, sd);
+    const int m1 = max(DN_M1, (int)ceilf((sqrtf(r8 * r8 + g * g) / DN_RHO + 3.5f) / 8.0f));
+    const int m2 = max(4, (int)ceilf((sqrtf(r32 * r32 + g * g) / DN_RHO + 15.5f) / 32.0f));
     if (m1 <= DN_M1_MAX) {
       p = {DN_REAL, m1, 0, m2, 1.0f, 0};
     } else if (8 * (DN_M1_MAX - 1) > reach) {    // the near window holds every line's points
@@ -280,18 +303,19 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
       float d8 = 0.0f, d32 = 0.0f;               // squared distances from which the complex moments hold
       for (int q = 0; q < bn.n; ++q) {
         const float gc = bn.c[q] * scale, e2 = bn.eta * bn.eta * gc * gc;
-        d8 = fmaxf(d8, (16.0f + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
-        d32 = fmaxf(d32, (256.0f + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
+        d8 = fmaxf(d8, (c8 * c8 + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
+        d32 = fmaxf(d32, (c32 * c32 + e2) / (DN_RHOC * DN_RHOC) - gc * gc);
       }
       p.kind = DN_COMPLEX;
       p.m1 = d8 > 0.0f ? (int)ceilf((sqrtf(d8) + 3.5f) / 8.0f) : 0;
       p.mh = d32 > 0.0f ? (int)ceilf((sqrtf(d32) + 15.5f) / 32.0f) : 0;
       p.m2 = max(m2, p.mh);
       // the moments of the divided blocks' groups are about the real centre
-      p.lines = sqrtf(16.0f + g * g) > DN_RHO_EDGE * (float)(reach - 8);
+      p.lines = sqrtf(r8 * r8 + g * g) > DN_RHO_EDGE * (float)(reach - 8);
+      if (p.m1 > DN_M1_MAX) p.kind = DN_NONE;
     }
     // lengths up to sqrt(16^2 + g^2): their 14th powers times a strength stay in range
-    p.ih = exp2f(-ceilf(0.5f * log2f(256.0f + g * g)));
+    p.ih = exp2f(-ceilf(0.5f * log2f(c32 * c32 + g * g)));
   }
   plan[c] = p;
 }
@@ -926,10 +950,10 @@ bool bartop::dense_applies(const bart_linelist& lines, const bart_nugrid& nu, do
   if (!(lo > 0.0)) return false;
   bool any = false;
   for (int c = 0; c < n_cells; ++c) {
-    // x of one grid interval: |x| >= 9 at the 8 m1 - 3.5 - 4 >= 24.5 points that
-    // a mid block's lines are away at least keeps the moments' asymptotic series
-    // below 1e-6; the near window's products of four squared x (within 12
-    // points of a line's) stay in the FP32 range
+    // x of one grid interval: from 0.4 on (a Doppler deviation of 1.8 points) the
+    // reach of a line's moments (dense_plan_kernel) stays within the near radii;
+    // the near window's products of four squared x (within 12 points of a
+    // line's) stay in the FP32 range
     const double dx_min = nu.dnu_cm / (hi * cells[c].dfac), dx_max = nu.dnu_cm / (lo * cells[c].dfac);
     cells[c].dense = dx_min >= 0.4 && dx_max <= 3000.0;
     any = any || cells[c].dense;
@@ -987,7 +1011,9 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
   dense_first_group_kernel<<<nb / 256 + 1, 256, 0, s>>>(lstart, range, gid, total, nb, gfirst);
   dense_point_kernel<<<(n_nu + 255) / 256, 256, 0, s>>>(win, jlo, jhi, range, gid, total, lstart, boff, nb, n_nu, pts);
   dense_gamma_kernel<<<std::min(tiles, 4 * ctx->sm_count), 256, 0, s>>>(gref, n, stat);
-  dense_plan_kernel<<<(n_cells + 127) / 128, 128, 0, s>>>(cells, n_cells, stat, (float)(1.0 / nu.dnu_cm), reach, pl, bins);
+  const double hi = nu.nu_start_cm + (double)n_nu * nu.dnu_cm + cutoff;
+  dense_plan_kernel<<<(n_cells + 127) / 128, 128, 0, s>>>(cells, n_cells, stat, (float)(1.0 / nu.dnu_cm),
+                                                         (float)(hi / nu.dnu_cm * 0.70710678118654752), reach, pl, bins);
   if ((st = bart_check_launch(ctx, "dense opacity prologue")) != BART_OK) return st;
   DenseArgs a{};
   a.win = win;
