@@ -47,9 +47,11 @@
 // Gauss-Hermite form (a positive sum of Lorentzians: no cancellation; <= 3.6e-7
 // for |z| >= 9) from |x| = 9 on, the full profile closer in.  Per-lane sums
 // stay in shared memory over the block's lines and are folded into a TwoSum
-// pair every 8 chunks; dense_sum_kernel adds the near windows of the 2 m1 - 1
-// blocks around a point, then the moments.  No atomics: every sum has a fixed
-// order.
+// pair every 8 chunks; the moments of a block's lines and a point's sums over
+// blocks are folded the same way (FoldedSum), so that rounding does not grow with
+// the number of lines or blocks.  dense_sum_kernel adds the near windows of the
+// 2 m1 - 1 blocks around a point, then the moments.  No atomics: every sum has a
+// fixed order.
 //
 // Used (dense_applies, dense_plan_kernel) for lists of at least DN_DENSITY lines
 // per point, where blocks pay for their fixed cost, and for cells whose widths
@@ -62,7 +64,8 @@
 // Measured: one species of the 5e6-line grid (1.67e6 lines, 100,000 points), 10
 // layers over 1e-8 .. 100 bar x 20 temperatures: 169 ms line by line, 58 ms with
 // the 160 cells of widths up to 3 points here, 44 ms with widths up to a sixth of
-// the cutoff, 40 ms with the near points in packed pairs, 28 ms with all cells
+// the cutoff, 40 ms with the near points in packed pairs, 28.3 ms with all cells,
+// 28.8 ms with the moments' sums compensated
 // (100 us of the near kernel and 15 of the sums per Doppler cell, whose near
 // points' profiles bound it: 80% of the issue slots);
 // 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart: 2.59 ms and
@@ -456,9 +459,38 @@ struct DenseArgs {
   float* out;
 };
 
+// hi + lo += v, exactly but for the rounding of lo (TwoSum).
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
+  const float t = hi + v, bp = t - hi;
+  lo += (hi - (t - bp)) + (v - bp);
+  hi = t;
+}
+// A running sum of few terms, folded into a compensated pair now and then.
+struct FoldedSum {
+  float s = 0.0f, hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void fold() {
+    two_sum(hi, lo, s);
+    s = 0.0f;
+  }
+  __device__ __forceinline__ float total() {
+    fold();
+    return hi + lo;
+  }
+};
+// term(i) for i in [from, to), folding the sum every 16 of them.
+template <typename F>
+__device__ __forceinline__ void folded_range(int from, int to, FoldedSum& sum, F term) {
+  for (int i = from; i < to;) {
+    const int stop = min(i + 16, to);
+    for (; i < stop; ++i) term(i);
+    if (i < to) sum.fold();
+  }
+}
+
 struct NearShared {
   float4 acc[DN_WARPS][DN_WIN / 4][32];      // per lane, four neighbouring points
-  float group[DN_WARPS][DN_GROUPS][DN_P];
+  float group[DN_WARPS][DN_GROUPS * DN_P];
+  float2 folded[DN_WARPS][DN_GROUPS * DN_P]; // the groups' sums before the last fold, compensated pairs
   int list[DN_WARPS][64];                    // lines of a bin, being gathered
 };
 
@@ -482,9 +514,13 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
   const float centre = (float)((m1 - 1) * DN_B) + 3.5f;       // the block's centre in the window
   const bool check = 8 * m1 >= a.reach;                       // the window passes the cutoff
   float4 (*acc)[32] = sh.acc[warp];
-  float (*grp)[DN_P] = sh.group[warp];
+  float* grp = sh.group[warp];
+  float2* grp_folded = sh.folded[warp];
   for (int s = 0; s < steps; ++s) acc[s][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int q = lane; q < DN_GROUPS * DN_P; q += 32) grp[q / DN_P][q % DN_P] = 0.0f;
+  for (int q = lane; q < DN_GROUPS * DN_P; q += 32) {
+    grp[q] = 0.0f;
+    grp_folded[q] = make_float2(0.f, 0.f);
+  }
   __syncwarp();
   float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f};     // points lane, lane + 32, lane + 64 of the window
   // adds the lanes' sums of every point (32 different banks at a time) into the
@@ -500,9 +536,7 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
 #pragma unroll 8
         for (int i = 0; i < 32; ++i) v += p[((i + s) & 31) * 4];
       }
-      const float t = hi[q] + v, bp = t - hi[q];
-      lo[q] += (hi[q] - (t - bp)) + (v - bp);
-      hi[q] = t;
+      two_sum(hi[q], lo[q], v);
     }
     __syncwarp();
   };
@@ -559,7 +593,7 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
       }
       if (tail && g < DN_GROUPS) {
 #pragma unroll
-        for (int n = 0; n < DN_P; ++n) grp[g][n] += M[n];
+        for (int n = 0; n < DN_P; ++n) grp[g * DN_P + n] += M[n];
       }
       __syncwarp();
     }
@@ -636,6 +670,12 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     if (++chunks % DN_FOLD == 0 && base + 32 < l1) {
       fold();
       for (int s = 0; s < steps; ++s) acc[s][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int e = lane; e < DN_GROUPS * DN_P; e += 32) {
+        float2 v = grp_folded[e];
+        two_sum(v.x, v.y, grp[e]);
+        grp_folded[e] = v;
+        grp[e] = 0.0f;
+      }
       __syncwarp();
     }
   }
@@ -645,11 +685,17 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
   for (int q = 0; q < 3; ++q)
     if (lane + 32 * q < n_pts) a.window[at * DN_WIN + lane + 32 * q] = hi[q] + lo[q];
   // the groups' moments, and the block's from them
-  for (int e = lane; e < ng * DN_P; e += 32) a.mg[((int64_t)blockIdx.y * a.g_stride + g0) * DN_P + e] = grp[e / DN_P][e % DN_P];
+  for (int e = lane; e < ng * DN_P; e += 32)
+    a.mg[((int64_t)blockIdx.y * a.g_stride + g0) * DN_P + e] = grp_folded[e].x + (grp_folded[e].y + grp[e]);
   if (lane < DN_P) {
-    float t = 0.0f;
-    for (int g = 0; g < ng; ++g) t += grp[g][lane];
-    a.m8[at * DN_P + lane] = t;
+    float t = 0.0f, l = 0.0f;
+    for (int g = 0; g < ng; ++g) {
+      const float2 v = grp_folded[g * DN_P + lane];
+      two_sum(t, l, v.x);
+      two_sum(t, l, grp[g * DN_P + lane]);
+      l += v.y;
+    }
+    a.m8[at * DN_P + lane] = t + l;
   }
   if (plan.kind != DN_COMPLEX) return;
   // ---- moments about the complex centres, bin by bin; the bin's lines are
@@ -661,7 +707,8 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
 #pragma unroll
     for (int n = 0; n < DN_PC; ++n) M[n] = make_float2(0.f, 0.f);
     const float gc = bn.c[bin] * cc.gfac;
-    int have = 0;
+    float2 mine = make_float2(0.f, 0.f), low = mine;          // lane n: moment n, a compensated pair
+    int have = 0, taken = 0;                                  // taken: chunks of 32 since the last fold
     for (int base = l0; base < l1; base += 32) {
       const int next = base + lane;
       const bool in = next < l1 &&
@@ -702,18 +749,23 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
         have -= 32;
       } while (have > 0 && base + 32 >= l1);
       have = max(have, 0);
-    }
-    float2 mine = make_float2(0.f, 0.f);
+      if (++taken < DN_FOLD && base + 32 < l1) continue;
+      taken = 0;
+      float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int n = 0; n < DN_PC; ++n) {
+      for (int n = 0; n < DN_PC; ++n) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        M[n].x += __shfl_xor_sync(0xffffffffu, M[n].x, o);
-        M[n].y += __shfl_xor_sync(0xffffffffu, M[n].y, o);
+        for (int o = 16; o > 0; o >>= 1) {
+          M[n].x += __shfl_xor_sync(0xffffffffu, M[n].x, o);
+          M[n].y += __shfl_xor_sync(0xffffffffu, M[n].y, o);
+        }
+        if (lane == n) sum = M[n];
+        M[n] = make_float2(0.f, 0.f);
       }
-      if (lane == n) mine = M[n];
+      two_sum(mine.x, low.x, sum.x);
+      two_sum(mine.y, low.y, sum.y);
     }
-    if (lane < DN_PC) a.mc8[(at * DN_BINS + bin) * DN_PC + lane] = mine;
+    if (lane < DN_PC) a.mc8[(at * DN_BINS + bin) * DN_PC + lane] = make_float2(mine.x + low.x, mine.y + low.y);
   }
 }
 
@@ -830,7 +882,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
 
   // ---- blocks inside the point's cutoff [bl, br), outside the near ones
   const int PL = (p.bl + 3) >> 2, PR = p.br >> 2;            // parents inside it
-  float far = 0.0f, mid = 0.0f;
+  FoldedSum far, mid;
   if (plan.kind == DN_COMPLEX) {
     const DenseBins bn = *a.bins;
     const float scale = a.cells[cell].gfac * a.inv_dnu * plan.ih;
@@ -838,27 +890,27 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
     const float2* mc32 = a.mc32 + (int64_t)blockIdx.y * (a.nb / 4) * DN_BINS * DN_PC;
     // parents inside the cutoff: real centre far away, complex centres nearer
     const int u0 = __reduce_min_sync(0xffffffffu, PL), u1 = __reduce_max_sync(0xffffffffu, PR);
-    for (int P = u0; P < u1; ++P) {
+    folded_range(u0, u1, far, [&](int P) {
       const int m = abs(P - T);                  // the same for the warp
       const bool in = P >= PL && P < PR;
       const float D = dist32(P);
       if (m >= plan.m2) {
-        if (in) far += moment_sum(m32 + (int64_t)P * DN_P, D);
+        if (in) far.s += moment_sum(m32 + (int64_t)P * DN_P, D);
       } else if (m >= plan.mh) {
         for (int q = 0; q < bn.n; ++q)
-          if (in) far += complex_sum(mc32 + ((int64_t)P * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
+          if (in) far.s += complex_sum(mc32 + ((int64_t)P * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
       }
-    }
+    });
     // blocks of the parents closer than that, and those beside the parents
     auto blocks8 = [&](int b0, int b1) {
       const int v0 = __reduce_min_sync(0xffffffffu, b0 < b1 ? b0 : 0x7fffffff);
       const int v1 = __reduce_max_sync(0xffffffffu, b0 < b1 ? b1 : -0x7fffffff);
-      for (int b = v0; b < v1; ++b) {
+      folded_range(v0, v1, mid, [&](int b) {
         const bool in = b >= b0 && b < b1 && abs(b - t) >= plan.m1;
         const float D = dist8(b);
         for (int q = 0; q < bn.n; ++q)
-          if (in) mid += complex_sum(mc8 + ((int64_t)b * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
-      }
+          if (in) mid.s += complex_sum(mc8 + ((int64_t)b * DN_BINS + q) * DN_PC, D, bn.c[q] * scale);
+      });
     };
     const int c0 = max(4 * (T - plan.mh + 1), 4 * PL), c1 = min(4 * (T + plan.mh), 4 * PR);
     if (PL < PR) {
@@ -874,17 +926,21 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   const int PS = max(T + plan.m2, PL), rbeg = max(t + plan.m1, p.bl);
   {
     const int u0 = __reduce_min_sync(0xffffffffu, PL), u1 = __reduce_max_sync(0xffffffffu, PE);
-    for (int P = u0; P < u1; ++P)
-      if (P >= PL && P < PE) far += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
+    folded_range(u0, u1, far, [&](int P) {
+      if (P >= PL && P < PE) far.s += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
+    });
     const int v0 = __reduce_min_sync(0xffffffffu, PS), v1 = __reduce_max_sync(0xffffffffu, PR);
-    for (int P = v0; P < v1; ++P)
-      if (P >= PS && P < PR) far += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
+    far.fold();
+    folded_range(v0, v1, far, [&](int P) {
+      if (P >= PS && P < PR) far.s += moment_sum(m32 + (int64_t)P * DN_P, dist32(P));
+    });
   }
   auto blocks = [&](int b0, int b1) {                        // [b0, b1), possibly empty
     const int u0 = __reduce_min_sync(0xffffffffu, b0 < b1 ? b0 : 0x7fffffff);
     const int u1 = __reduce_max_sync(0xffffffffu, b0 < b1 ? b1 : -0x7fffffff);
-    for (int b = u0; b < u1; ++b)
-      if (b >= b0 && b < b1) mid += moment_sum(m8 + (int64_t)b * DN_P, dist8(b));
+    folded_range(u0, u1, mid, [&](int b) {
+      if (b >= b0 && b < b1) mid.s += moment_sum(m8 + (int64_t)b * DN_P, dist8(b));
+    });
   };
   const bool hasL = PE > PL, hasR = PR > PS;
   blocks(p.bl, hasL ? min(4 * PL, lend) : lend);
@@ -897,22 +953,23 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
   // within the near radius were taken line by line), or, where the profiles
   // are too wide for their moments about the real centre, line by line: at
   // least 23 points away, |x| > 9 (dense_applies), by the far form
-  float edge = 0.0f, direct = 0.0f;
+  float edge = 0.0f;                                         // (of 2 DN_GROUPS terms at most)
+  FoldedSum direct;
   const bool both = p.bl > p.br;                             // both edges divide the same block
   if (plan.lines) {
     const CellConst cc = a.cells[cell];
     const float ln_thr = a.smax ? ordered_float(a.smax[a.tmap[cell]]) + a.ln_rel : -3.0e38f;
     auto lines = [&](int i0, int i1, int b) {
       if (abs(b - t) < plan.m1) return;
-      for (int i = i0; i < i1; ++i) {
+      folded_range(i0, i1, direct, [&](int i) {
         const LineWin w = a.win[i];
         const float ln_s = line_ln_s(w, cc);
-        if (!(ln_s >= ln_thr)) continue;
+        if (!(ln_s >= ln_thr)) return;
         const float inv = bartw::rcp_approx(w.nu0f * cc.dfac), y = a.gref[i] * cc.gfac * inv;
         const float S = ex2f_approx((ln_s + LN_SCALE) * LOG2EF);
         const float x = fmaf((float)(j - w.jc), a.dnu * inv, w.delta * inv);
-        direct = fmaf(S * inv * bartw::INV_SQRTPI * (y * bartw::INV_SQRTPI), far_ratio(x, y * y), direct);
-      }
+        direct.s = fmaf(S * inv * bartw::INV_SQRTPI * (y * bartw::INV_SQRTPI), far_ratio(x, y * y), direct.s);
+      });
     };
     if (both) {
       lines(p.il, p.ir, p.br);
@@ -933,7 +990,7 @@ dense_sum_kernel(const __grid_constant__ DenseArgs a) {
       if (p.br < a.nb) groups(max(a.gfirst[p.br], p.gl), p.gr, p.br);
     }
   }
-  if (j0 + lane < a.n_nu) a.out[(int64_t)cell * a.n_nu + j] = (((edge + far) + mid) * plan.ih + (near + direct)) * INV_SCALE;
+  if (j0 + lane < a.n_nu) a.out[(int64_t)cell * a.n_nu + j] = (((edge + far.total()) + mid.total()) * plan.ih + (near + direct.total())) * INV_SCALE;
 }
 
 }  // namespace
