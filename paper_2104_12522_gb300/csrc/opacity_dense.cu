@@ -601,8 +601,9 @@ dense_near_kernel(const __grid_constant__ DenseArgs a) {
     // ---- near points.  The warp's lines lie in [cmin, cmax] (window
     // coordinates); a point's smallest |x| over them decides the form.
     const float pos = off - w.delta * a.inv_dnu;
-    const float cmin = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(pos)));
-    const float cmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(pos)));
+    // (a window of one block has lines up to half a point left of its first point)
+    const float cmin = ordered_float(__reduce_min_sync(0xffffffffu, ordered_int(pos)));
+    const float cmax = ordered_float(__reduce_max_sync(0xffffffffu, ordered_int(pos)));
     const float dxm = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(dx)));
     const float ymax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(y)));
     const float ymin = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(y)));
