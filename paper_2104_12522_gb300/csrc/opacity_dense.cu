@@ -6,7 +6,7 @@
 // 2,500 points, so most of the work of a line-by-line sum is far wings of lines
 // that lie within a fraction of a point of one another.  Lines are taken in
 // source blocks of 8 grid points (by their nearest point jc).  For a point j
-//   near   source blocks closer than m1 blocks: every line evaluated on its own
+//   near   source blocks closer than m1 (5) blocks: every line evaluated on its own
 //          (dense_near_kernel);
 //   mid    source blocks from m1 blocks on, by their moments;
 //   far    blocks of 32 points from m2 such blocks on, by theirs;
@@ -55,7 +55,7 @@
 //
 // Used (dense_applies, dense_plan_kernel) for lists of at least DN_DENSITY lines
 // per point, where blocks pay for their fixed cost, and for cells whose widths
-// fit: Doppler widths that keep |x| >= 9 from the first mid block on; Lorentz
+// fit: Doppler deviations up to 1.8 grid points (x of an interval 0.4); Lorentz
 // widths up to about 3 grid points, or gamma_ref within a factor 4 over the
 // list (4 bins), or a cutoff so short that the near window holds all of it.
 // Other cells go line by line.  From a sixth of the cutoff on a divided block's
@@ -65,11 +65,10 @@
 // layers over 1e-8 .. 100 bar x 20 temperatures: 169 ms line by line, 58 ms with
 // the 160 cells of widths up to 3 points here, 44 ms with widths up to a sixth of
 // the cutoff, 40 ms with the near points in packed pairs, 28.3 ms with all cells,
-// 28.8 ms with the moments' sums compensated
-// (100 us of the near kernel and 15 of the sums per Doppler cell, whose near
-// points' profiles bound it: 80% of the issue slots);
-// 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart: 2.59 ms and
-// 0.31 ms.
+// 28.8 ms with the moments' sums compensated (100 us of the near kernel and 17 of
+// the sums per Doppler cell, whose near points' profiles bound it: 80% of the
+// issue slots); 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart:
+// 2.59 ms and 0.32 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -81,14 +80,17 @@ namespace {
 
 constexpr int DN_B = 8;                     // points of a source block
 constexpr int DN_P = 8;                     // moments
-constexpr int DN_M1 = 4, DN_M1_MAX = 5;     // near radius in blocks
-constexpr int DN_WIN = (2 * DN_M1_MAX - 1) * DN_B;   // near points of a block, at most
+constexpr int DN_M1 = 5;                    // near radius in blocks about real centres (a mid block's centre is 36.5
+                                            // points away; 4 blocks, 28.5 points, would not do for a half width of 4),
+                                            // and the largest about complex ones
+constexpr int DN_WIN = (2 * DN_M1 - 1) * DN_B;   // near points of a block, at most
 constexpr int DN_GROUPS = 20;               // groups of a block: jlo and jhi each step at most 9 times
 constexpr float DN_RHO = 0.14f;
 constexpr int DN_BINS = 4;                  // bins of gamma_ref
 constexpr int DN_PC = 14;                   // moments about a complex centre
 constexpr float DN_RHOC = 0.305f;
-constexpr float DN_RHO_EDGE = 0.175f;       // divided blocks: 9 x 0.175^8 = 8e-6 of a line at its cutoff
+constexpr float DN_RHO_EDGE = 0.175f;       // divided blocks: 9e-7 of a line at its cutoff (against the Faddeeva
+                                            // function in 64 bits; 9 x 0.175^8 = 8e-6 would be a half width's share)
 constexpr double DN_DENSITY = 0.5;          // lines per point
 constexpr int DN_WARPS = 4;
 constexpr int DN_FOLD = 8;                  // chunks of 32 lines between two folds
@@ -296,12 +298,10 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
     // a point of block t is at least 8 m - 3.5 points from the centre of block t +- m
     const float sd = sigma * cells[c].dfac;
     const float r8 = reach8(4.0f, sd), r32 = reach8(16.0f, sd), c8 = reach14(4.0f, sd), c32 = reach14(16.0f, sd);
-    const int m1 = max(DN_M1, (int)ceilf((sqrtf(r8 * r8 + g * g) / DN_RHO + 3.5f) / 8.0f));
     const int m2 = max(4, (int)ceilf((sqrtf(r32 * r32 + g * g) / DN_RHO + 15.5f) / 32.0f));
-    if (m1 <= DN_M1_MAX) {
-      p = {DN_REAL, m1, 0, m2, 1.0f, 0};
-    } else if (8 * (DN_M1_MAX - 1) > reach) {    // the near window holds every line's points
-      p = {DN_REAL, DN_M1_MAX, 0, m2, 1.0f, 0};
+    if (sqrtf(r8 * r8 + g * g) <= DN_RHO * (8.0f * DN_M1 - 3.5f) ||
+        8 * (DN_M1 - 1) > reach) {               // (or the near window holds every line's points)
+      p = {DN_REAL, DN_M1, 0, m2, 1.0f, 0};
     } else if (bn.n > 0) {
       float d8 = 0.0f, d32 = 0.0f;               // squared distances from which the complex moments hold
       for (int q = 0; q < bn.n; ++q) {
@@ -315,7 +315,7 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
       p.m2 = max(m2, p.mh);
       // the moments of the divided blocks' groups are about the real centre
       p.lines = sqrtf(r8 * r8 + g * g) > DN_RHO_EDGE * (float)(reach - 8);
-      if (p.m1 > DN_M1_MAX) p.kind = DN_NONE;
+      if (p.m1 > DN_M1) p.kind = DN_NONE;
     }
     // lengths up to sqrt(16^2 + g^2): their 14th powers times a strength stay in range
     p.ih = exp2f(-ceilf(0.5f * log2f(c32 * c32 + g * g)));
@@ -1025,8 +1025,8 @@ bart_status bartop::dense_cells(bart_ctx* ctx, const LineWin* win, const int* jl
                                 const DensePlan** plan) {
   const int n_nu = (int)nu.n_nu, n = (int)n_lines;
   const int reach = (int)std::floor(cutoff / nu.dnu_cm);
-  const int boff = ((reach + 2) / DN_B + DN_M1_MAX + 4) / 4 * 4;         // blocks before the grid, whole parents
-  const int nb = (boff + n_nu / DN_B + (reach + 2) / DN_B + DN_M1_MAX + 8) / 4 * 4;
+  const int boff = ((reach + 2) / DN_B + DN_M1 + 4) / 4 * 4;         // blocks before the grid, whole parents
+  const int nb = (boff + n_nu / DN_B + (reach + 2) / DN_B + DN_M1 + 8) / 4 * 4;
   const int tiles = (n + GR_TILE - 1) / GR_TILE;
   const int64_t g_max = std::min<int64_t>(n, (int64_t)nb * DN_GROUPS) + 1;
   const size_t per_cell = ((size_t)nb * (DN_WIN + DN_P) + (size_t)(nb / 4) * DN_P + (size_t)g_max * DN_P +
