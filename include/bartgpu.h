@@ -98,8 +98,8 @@ bart_status bart_set_emission_tile(bart_ctx* ctx, int tile);
  *     A CTA thread takes two wavenumbers and their arithmetic runs on packed
  *     FP32 pairs; four where nu.n_nu is a multiple of 4, the grid is 16-byte
  *     aligned and the call large (24 entries or more that fill the SMs twice).
- *     From 10 entries per grid temperature on, without spans and mask, such a
- *     call first checks the whole grid: if every opacity is finite and not
+ *     From 10 entries per grid temperature (and 1e8 grid values to read in
+ *     all) on, without spans and mask, such a call first checks the whole grid: if every opacity is finite and not
  *     negative, columns end at the level below which nothing changes their
  *     fluxes (the bits are those of all levels).  It addresses grid rows by 32-bit element offsets: grids
  *     with n_species * n_layers * n_temps * n_nu + n_nu >= 2^32 (16 GiB and

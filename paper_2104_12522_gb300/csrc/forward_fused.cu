@@ -66,8 +66,12 @@ grid_check_kernel(const float* __restrict__ grid, size_t n, int* __restrict__ ba
 // Proposals per grid temperature from which a call checks the grid so that
 // columns may end early.  The check reads S L M n_nu values from DRAM (3.2 GB:
 // 0.48 ms); the layers that n proposals leave out save 0.40 ms of 128 proposals
-// on a grid of 20 temperatures, 0.78 ms of 256, 1.5 ms of 512.
+// on a grid of 20 temperatures, 0.78 ms of 256, 1.5 ms of 512.  Of the smallest
+// grids its two launches are the cost, 6 us (200 x 60 x 4,096, 2 species: 102 us
+// without, 110 with; 100 x 100 x 8,000, 4 species: 172 and 165): n S L n_nu of at
+// least CHECK_VALUES.
 constexpr int CHECK_FROM = 10;
+constexpr double CHECK_VALUES = 1e8;
 
 }  // namespace
 
@@ -98,8 +102,8 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   const int mode = emission_mode(g, c);
   // columns may end early where the grid was checked (by the retrieval loop) or
   // the check pays for the call (of which every proposal is active)
-  const bool ends =
-      (ctx->grid_bad || (n >= (int64_t)CHECK_FROM * M && !b->active)) && columns_may_end(ctx, g, c, b);
+  const bool pays = n >= (int64_t)CHECK_FROM * M && (double)n * S * L * (double)N >= CHECK_VALUES && !b->active;
+  const bool ends = (ctx->grid_bad || pays) && columns_may_end(ctx, g, c, b);
   const FusedForm form = fused_form(ctx, g, n, ends);
   if (S > FUSED_MAX_SPECIES || !pick_fused(S, NA, form, FUSED_THREADS[1], mode))
     return bart_fail(ctx, BART_EUNSUPPORTED, "emission with %d species and %d angles is not instantiated "
