@@ -65,9 +65,9 @@
 // layers over 1e-8 .. 100 bar x 20 temperatures: 169 ms line by line, 58 ms with
 // the 160 cells of widths up to 3 points here, 44 ms with widths up to a sixth of
 // the cutoff, 40 ms with the near points in packed pairs, 28.3 ms with all cells,
-// 28.8 ms with the moments' sums compensated (100 us of the near kernel and 17 of
-// the sums per Doppler cell, whose near points' profiles bound it: 80% of the
-// issue slots); 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart:
+// 28.8 ms with the moments' sums compensated (100 to 170 us of the near kernel
+// and 15 of the sums per cell; the near kernel's per-lane sums in shared memory
+// and its profiles bound it: L1 data pipe 87%, issue 53% of the slots at 0.1 bar); 2 species x 10,000 lines, 60 cells, 2,000 points 1 cm^-1 apart:
 // 2.59 ms and 0.32 ms.
 #include <algorithm>
 #include <cmath>
@@ -324,7 +324,7 @@ __global__ void dense_plan_kernel(const CellConst* __restrict__ cells, int n_cel
 }
 
 // Pairs of points in packed FP32 (one issue slot for both; the near kernel is
-// bound by issue).
+// bound by its instructions and its sums in shared memory).
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
