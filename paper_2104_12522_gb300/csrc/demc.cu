@@ -689,10 +689,10 @@ series_centre_kernel(const float* __restrict__ chain, int n, int64_t ld, int64_t
 // are few series or their memories differ; a CTA leaves once a lag below its
 // chunk has fallen below the threshold (first[], atomicMin), so every lag
 // before the first crossing is always written.
-// Measured, 20,000 x 16 chains x 9 parameters with about 700 lags a series:
-// 101 ms with a CTA per series subtracting and converting from the strided
-// chain at every lag and the Gelman-Rubin sums in one thread per chain, 7.4 ms
-// now (the FP64 FMAs alone need 3.2 ms).
+// Measured, 20,000 x 16 chains x 9 parameters with about 700 lags a series: 73
+// to 101 ms (by the series' memories) with a CTA per series subtracting and
+// converting from the strided chain at every lag and the Gelman-Rubin sums in
+// one thread per chain, 6.7 to 9.0 ms now (the FP64 FMAs alone need 3.2 ms).
 constexpr int LG_LAGS = 4;
 constexpr int LG_CHUNK = LG_LAGS * ST_THREADS / 32;
 
