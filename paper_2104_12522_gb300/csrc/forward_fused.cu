@@ -118,10 +118,12 @@ bart_status bartem::fused_emission(bart_ctx* ctx, const bart_grid_desc* g, const
   void *p_const, *p_work, *p_done = nullptr, *p_part = nullptr;
   if ((st = bart_upload_const(ctx, "ff_const", hconst.data(), hconst.size() * sizeof(float), &p_const)) != BART_OK)
     return st;
-  void *p_twc, *p_flag;
+  void *p_twc, *p_flag, *p_bad;
   if ((st = bart_scratch(ctx, "ff_work", 3 * sizeof(unsigned long long), &p_work)) != BART_OK) return st;
   if ((st = bart_scratch(ctx, "ff_twc", (size_t)n * L * sizeof(LayerTW), &p_twc)) != BART_OK) return st;
   if ((st = bart_scratch(ctx, "ff_flag", (size_t)n * sizeof(unsigned int), &p_flag)) != BART_OK) return st;
+  // (of every call, so that a capture may follow an eager call that did not check)
+  if ((st = bart_scratch(ctx, "ff_bad", sizeof(int), &p_bad)) != BART_OK) return st;
   const int max_tiles = (int)((N + 3 + 2 * FUSED_THREADS[0] - 1) / (2 * FUSED_THREADS[0]));   // smallest tile, aligned start
   if (nb > 0) {
     if ((st = bart_scratch(ctx, "ff_done", (size_t)n * sizeof(unsigned int), &p_done)) != BART_OK) return st;

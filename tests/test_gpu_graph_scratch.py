@@ -61,3 +61,28 @@ def test_dense_opacity_after_calls_with_longer_cutoffs():
         ctx.sync()
 
     _replays(ctx, lambda: ctx.opacity_cells(lists, p, t, nu, 5.0, out=out), out, larger)
+
+
+def test_capture_after_an_eager_call_with_a_mask():
+    """A masked call needs no check of the grid, the unmasked one of the same shape does: its capture needs no
+    eager call of its own."""
+    import torch
+    import paper_2104_12522_gb300 as bart
+    ctx = make_ctx()
+    S, L, N, n = 2, 60, 1024, 1000
+    p = W.log_pressures(L, 1e-8, 100.0)
+    cfg = dict(geometry=0, n_angles=4, g=W.HD189_GRAV_CGS, mu=2.3, x0=[W.BASE_VMR] * S, t_int=W.T_INT_K,
+               t_star=W.HD189_TSTAR_K, r_star_tp=W.HD189_RSTAR_CM, a_orbit=W.HD189_A_CM, t_min=500.0, t_max=3000.0)
+    grid = torch.tensor(W.opacity_field(S, p, np.array([500.0, 3000.0]), N, seed=9)[:, :, :1].copy(), device="cuda")
+    theta = torch.tensor(W.proposals(n, n_species=S), device="cuda")
+    spec, nu = torch.zeros((n, N), device="cuda"), bart.NuGrid(1000.0, 0.05, N)
+    call = lambda **kw: ctx.forward_spectra_batch(grid, p, [1000.0], nu, cfg, theta=theta, spectra=spec, **kw)
+    call(active=torch.ones(n, dtype=torch.int32, device="cuda"))
+    ctx.sync()
+    want = spec.clone()
+    g = ctx.capture(call)
+    spec.zero_()
+    torch.cuda.synchronize()
+    g.launch()
+    ctx.sync()
+    assert torch.equal(spec, want)
