@@ -817,12 +817,12 @@ extern "C" bart_status bart_chain_stats(bart_ctx* ctx, const float* chain, int n
   const int rows = std::max(64, (int)(((int64_t)n + ST_MAX_CHUNKS - 1) / ST_MAX_CHUNKS));
   const int n_chunks = (int)(((int64_t)n + rows - 1) / rows);
   // Series are taken in batches whose memory (12 n bytes a series for the lag
-  // sums: the centred series and the autocorrelations) stays within 512 MB,
+  // sums: the centred series and the autocorrelations; 16 per chunk) stays within 512 MB,
   // at least one series at a time, and in smaller ones where that is not free.
   // It belongs to this call alone: calls on other streams of the context and
   // graphs that captured one are independent of it.
-  const int64_t per = (int64_t)n * 8 + (int64_t)(n / 2) * 8;
-  int batch = (int)std::min<int64_t>(series, std::max<int64_t>(1, speis ? (512LL << 20) / per : 1 << 20));
+  const int64_t per = 16LL * n_chunks + (speis ? (int64_t)n * 8 + (int64_t)(n / 2) * 8 : 0);
+  int batch = (int)std::min<int64_t>(series, std::max<int64_t>(1, (512LL << 20) / per));
   bart_status st;
   double *sums = nullptr, *sq = nullptr, *e = nullptr, *rho = nullptr, *tot = nullptr;
   int* first = nullptr;
